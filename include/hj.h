@@ -128,7 +128,7 @@ typedef struct {
     double t_final;        /* simulated time reached */
     double dt_first;       /* dt of the first step of this call (0 if none) */
     double dt_last;        /* dt of the last step of this call (0 if none) */
-    double alpha_max[4];   /* alpha_d^max reduced by the last step (|xdot_d| maxima) */
+    double alpha_max[4];   /* alpha_d^max of the dynamics over the grid (|xdot_d| maxima) */
     double device_ms;      /* device time of the whole call (CUDA events) */
     double loop_ms;        /* device time of the time loop only (step kernels) */
     int32_t kernel;        /* hj_kernel actually used */

@@ -3,10 +3,10 @@
 // Host side of the HJ reachability solver for arxiv 2012.04011: grid and
 // buffer management, the (v, theta) state tables (Sec. III-A), V0 ingest,
 // the time loop driving the step kernels (Algorithms 1-2, Sec. II-B), and
-// readback.  Simulated time and dt live on the device in FP64 and are
-// advanced by the step kernels themselves (fused alpha^max reduction and
-// finaliser, hj_device.cuh); the host only launches steps and reads the
-// state back to know when the horizon is reached.
+// readback.  The time loop runs here, in FP64: alpha^max of every supported
+// dynamics does not depend on V (the paper's remark that dt can be
+// precomputed, Sec. II-B), so t, dt and the step count are known before the
+// steps run, and a solve queues all of them and waits once.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -81,7 +81,7 @@ __global__ void ingest_kernel(const Tin *__restrict__ src, T *__restrict__ dst, 
         }
         dst[i] = v;
     }
-    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(nonfinite, 1);
+    if (__syncthreads_or(bad) && threadIdx.x == 0) *(volatile int *)nonfinite = 1;
 }
 
 // V0 that depends only on (x, y): an N1*N2 field replicated over v and theta
@@ -104,7 +104,7 @@ __global__ void ingest_xy_kernel(const Tin *__restrict__ src, T *__restrict__ ds
         }
         dst[i] = v;
     }
-    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(nonfinite, 1);
+    if (__syncthreads_or(bad) && threadIdx.x == 0) *(volatile int *)nonfinite = 1;
 }
 
 // Internal layout -> dense (rows [row0, row0 + nrows)), converting type.
@@ -121,28 +121,44 @@ __global__ void readback_kernel(const T *__restrict__ src, Tout *__restrict__ ds
     }
 }
 
-// Start of a solve call: horizon, Courant number and the dt of the first
-// step.  Right after V0 is set (n == 0), alpha^max is reduced over the
-// (v, theta) table, which holds |xdot_1|, |xdot_2| of every cell (the car's
-// velocity depends only on v and theta).
-template <typename T>
-__global__ void prologue_kernel(HjDevState *st, const HjGeom g, const HjCoef<T> *__restrict__ coef, int ncoef,
-                                double T_end, double cfl, HjScaledCoef *scaled = nullptr, int32_t *qw = nullptr,
-                                const double *k4 = nullptr, double threshold = 0.0)
+// Start of a solve call: the step sizes and the convergence mode's state
+// into the device constants and, for FP64 / Q5.27 grids, the dt-scaled tables
+// (build[i]: table i is not the one of dt[i] yet).
+struct PrologueArgs {
+    double dt[2], threshold;
+    int build[2];
+};
+
+__global__ void prologue_kernel(HjLoop *lp, const PrologueArgs a, const HjGeom g,
+                                const HjCoef<double> *__restrict__ coef, HjScaledCoef *scaled, int32_t *qw,
+                                const double *__restrict__ k4)
+{
+    const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    if (first == 0) {
+        lp->dt[0] = a.dt[0];
+        lp->dt[1] = a.dt[1];
+        lp->threshold = a.threshold;
+        lp->delta_last = 0.0;
+        lp->delta_bits = 0ull;
+        lp->taken = 0;
+        lp->done = 0;
+        lp->blocks_done = 0u;
+    }
+    for (int i = 0; i < 2; ++i) {
+        if (!a.build[i]) continue;
+        if (scaled) hj_rescale_table(scaled + (size_t)i * g.n3 * g.n4, coef, k4, g.n3, g.n4, a.dt[i], first, stride);
+        else if (qw)
+            hj_rescale_qweights(qw + i * hj_qw_count(g.n3, g.p4), coef, g.n3, g.n4, g.p4, g.k3, k4, a.dt[i], first,
+                                stride);
+    }
+}
+
+// Start of a batch slot's solve (the slot's time loop runs on the device).
+__global__ void slot_prologue_kernel(HjDevState *st, const HjGeom g, const HjCoef<float> *__restrict__ coef, int ncoef,
+                                     double T_end, double cfl)
 {
     __shared__ unsigned long long scratch[64];
-    hj_prologue_block(st, g, coef, ncoef, T_end, cfl, threshold, scratch);
-    if (scaled || qw) {  // FP64 / Q5.27 grids: the dt-scaled tables must match the first dt
-        __syncthreads();
-        const volatile HjDevState *vs = st;
-        const double dt = vs->dt;
-        if (!vs->done && dt != vs->dt_scaled) {
-            if (scaled) hj_rescale_table(scaled, (const HjCoef<double> *)coef, k4, g.n3, g.n4, dt);
-            else hj_rescale_qweights(qw, (const HjCoef<double> *)coef, g.n3, g.n4, g.p4, g.k3, k4, dt);
-            __syncthreads();
-            if (threadIdx.x == 0) st->dt_scaled = dt;
-        }
-    }
+    hj_prologue_block(st, g, coef, ncoef, T_end, cfl, scratch);
 }
 
 int grid_blocks(long long work, int threads)
@@ -173,12 +189,16 @@ hj_status activate(const hj_grid *g)
     return HJ_OK;
 }
 
-hj_status pull_state(hj_grid *g)
+// Waits for the grid's stream: everything queued has run and the host flags
+// are current.
+hj_status wait_stream(const hj_grid *g)
 {
-    HJ_CUDA(cudaMemcpyAsync(g->hstate, g->dstate, sizeof(HjDevState), cudaMemcpyDeviceToHost, g->stream));
     HJ_CUDA(cudaStreamSynchronize(g->stream));
     return HJ_OK;
 }
+
+// The flags, as the host reads them after a synchronisation.
+int read_status(const hj_grid *g) { return *(volatile int *)&g->hflags->status; }
 
 hj_status upload_tables(hj_grid *g)
 {
@@ -271,27 +291,15 @@ hj_status upload_tables(hj_grid *g)
                                    cudaMemcpyHostToDevice);
         if (e != cudaSuccess) st = set_err(HJ_ERR_CUDA, "table upload: %s", cudaGetErrorString(e));
     }
-    // the largest |xdot_1|, |xdot_2| over each theta quad's real headings, per speed
-    if (st == HJ_OK) {
-        const int Q4 = P4 / 4;
-        double2 *aq = (double2 *)malloc(sizeof(double2) * (size_t)N3 * Q4);
-        if (!aq) st = set_err(HJ_ERR_OOM, "host allocation failed");
-        for (int k = 0; aq && k < N3; ++k)
-            for (int q = 0; q < Q4; ++q) {
-                double m1 = 0.0, m2 = 0.0;
-                for (int l = 4 * q; l < 4 * q + 4 && l < N4; ++l) {
-                    const double a1 = fabs(f1[(size_t)k * N4 + l]), a2 = fabs(f2[(size_t)k * N4 + l]);
-                    if (a1 > m1) m1 = a1;
-                    if (a2 > m2) m2 = a2;
-                }
-                aq[(size_t)k * Q4 + q] = make_double2(m1, m2);
-            }
-        if (aq) {
-            cudaError_t e = cudaMemcpy(g->amax_q, aq, sizeof(double2) * (size_t)N3 * Q4, cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) st = set_err(HJ_ERR_CUDA, "table upload: %s", cudaGetErrorString(e));
-        }
-        free(aq);
+    // alpha^max over the grid's (v, theta) states (FP64 in every precision, so
+    // that the dt sequence of Algorithm 1 is the FP64 one)
+    g->alpha[0] = g->alpha[1] = 0.0;
+    for (size_t i = 0; i < nco; ++i) {
+        if (fabs(f1[i]) > g->alpha[0]) g->alpha[0] = fabs(f1[i]);
+        if (fabs(f2[i]) > g->alpha[1]) g->alpha[1] = fabs(f2[i]);
     }
+    g->alpha[2] = g->geom.alpha3;  // |a_opt| = a_max at every cell (bang-bang), |c3| for constant dynamics
+    g->alpha[3] = g->geom.alpha4;
     free(f1);
     free(f2);
     free(tab);
@@ -300,12 +308,13 @@ hj_status upload_tables(hj_grid *g)
     return st;
 }
 
-hj_status reset_state(hj_grid *g)
+// Back to t = 0 (the stream is idle: every call waits for its own work).
+void reset_state(hj_grid *g)
 {
-    memset(g->hstate, 0, sizeof(HjDevState));
-    g->hstate->status = HJ_OK;
-    HJ_CUDA(cudaMemcpyAsync(g->dstate, g->hstate, sizeof(HjDevState), cudaMemcpyHostToDevice, g->stream));
-    return HJ_OK;
+    g->t = 0.0;
+    g->nstep = 0;
+    g->hflags->status = HJ_OK;
+    g->hflags->nonfinite = 0;
 }
 
 // Whether HJ_KERNEL_AUTO takes the resident kernel: FP32 grids of up to 4 M
@@ -328,11 +337,9 @@ hj_kernel effective_kernel(const hj_grid *g)
     return g->tiled_ok ? HJ_KERNEL_TILED : HJ_KERNEL_GENERIC;
 }
 
-hj_status launch_step(hj_grid *g, hj_kernel k)
+hj_status launch_step(hj_grid *g, hj_kernel k, long long n, int sel)
 {
-    cudaError_t e = (k == HJ_KERNEL_TILED)     ? hj_launch_step_tiled(g)
-                    : (k == HJ_KERNEL_RESIDENT) ? hj_launch_step_resident(g, 1)
-                                                : hj_launch_step_generic(g);
+    cudaError_t e = (k == HJ_KERNEL_TILED) ? hj_launch_step_tiled(g, n, sel) : hj_launch_step_generic(g, n, sel);
     if (e != cudaSuccess) {
         cudaGetLastError();  // a failed call (not a sticky fault) must not fail later checks
         return set_err(e == cudaErrorMemoryAllocation ? HJ_ERR_OOM : HJ_ERR_CUDA, "step launch: %s",
@@ -345,19 +352,21 @@ hj_status launch_step(hj_grid *g, hj_kernel k)
 // launching it costs, so their time loop replays captured graphs.
 constexpr long long GRAPH_MAX_CELLS = 1LL << 24;
 
-// k step launches as one graph launch (captured on first use, kept in a
-// 4-entry cache); false if a graph cannot be used here (the stream is being
-// captured by the caller, or capture failed), and the caller launches the
-// steps one by one.
-bool launch_steps_graph(hj_grid *g, hj_kernel kern, long long k)
+// k step launches from V after n steps (the last one cut to the horizon if
+// cut) as one graph launch (captured on first use, kept in a 4-entry cache);
+// false if a graph cannot be used here (the stream is being captured by the
+// caller, or capture failed), and the caller launches the steps one by one.
+bool launch_steps_graph(hj_grid *g, hj_kernel kern, long long n, long long k, bool cut)
 {
+    const int parity = n == 0 ? 0 : 1 + (int)((n - 1) & 1);
     if (g->ncell >= GRAPH_MAX_CELLS || k < 4 || k > 4096) return false;
     cudaStreamCaptureStatus cs;
     if (cudaStreamIsCapturing(g->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
     int hit = -1, victim = 0;
     for (int i = 0; i < 4; ++i) {
         const hj_grid::StepGraph &e = g->graphs[i];
-        if (e.exec && e.k == k && e.kernel == (int)kern && e.track == (int)g->track && e.version == g->launch_version)
+        if (e.exec && e.k == k && e.kernel == (int)kern && e.track == (int)g->track && e.cut == (int)cut &&
+            e.parity == parity && e.version == g->launch_version)
             hit = i;
         if (!g->graphs[i].exec) victim = i;
     }
@@ -374,8 +383,11 @@ bool launch_steps_graph(hj_grid *g, hj_kernel kern, long long k)
             return false;
         }
         bool ok = true;
-        for (long long i = 0; i < k && ok; ++i)
-            ok = ((kern == HJ_KERNEL_TILED) ? hj_launch_step_tiled(g) : hj_launch_step_generic(g)) == cudaSuccess;
+        for (long long i = 0; i < k && ok; ++i) {
+            const int sel = cut && i == k - 1;
+            ok = ((kern == HJ_KERNEL_TILED) ? hj_launch_step_tiled(g, n + i, sel)
+                                            : hj_launch_step_generic(g, n + i, sel)) == cudaSuccess;
+        }
         const cudaError_t ce = cudaStreamEndCapture(g->stream, &graph);
         if (!ok || ce != cudaSuccess || !graph) {
             if (graph) cudaGraphDestroy(graph);
@@ -392,6 +404,8 @@ bool launch_steps_graph(hj_grid *g, hj_kernel kern, long long k)
         e.k = k;
         e.kernel = (int)kern;
         e.track = (int)g->track;
+        e.cut = (int)cut;
+        e.parity = parity;
         e.version = g->launch_version;
         hit = victim;
     }
@@ -410,18 +424,38 @@ void with_elem(hj_precision p, F &&f)
 
 bool valid_prec(hj_precision p) { return p == HJ_FP64 || p == HJ_FP32 || p == HJ_Q527; }
 
-// Start of a solve call (horizon, Courant number, first dt, and the FP64 /
-// fixed-point tables scaled for it).
-void launch_prologue(hj_grid *g, double T, double cfl, double threshold = 0.0)
+// Algorithm 1's step size, dt = CFL / sum_d alpha_d^max / dx_d, in the
+// oracle's FP64 operations and order; false if it is not a usable number.  A
+// sum of 0 gives dt = 0 (one step to the horizon).
+bool cfl_step(const hj_grid *g, double cfl, double *dt)
 {
-    const int ncoef = g->n[2] * g->n[3];
-    if (g->prec == HJ_FP32)
-        prologue_kernel<float><<<1, 256, 0, g->stream>>>(g->dstate, g->geom, (const HjCoef<float> *)g->coef, ncoef, T,
-                                                         cfl, nullptr, nullptr, nullptr, threshold);
-    else
-        prologue_kernel<double><<<1, 256, 0, g->stream>>>(g->dstate, g->geom, (const HjCoef<double> *)g->coef, ncoef,
-                                                          T, cfl, g->scaled, g->qw, (const double *)g->k4tab,
-                                                          threshold);
+    double S = 0.0;
+    for (int d = 0; d < 4; ++d) S = S + g->alpha[d] / g->h[d];
+    *dt = S == 0.0 ? 0.0 : cfl / S;
+    return *dt >= 0.0 && !isinf(*dt);
+}
+
+// Step sizes dt0 (regular) and dt1 (cut to the horizon) for the steps queued
+// next.  Nothing is launched when the device already holds them.
+hj_status launch_prologue(hj_grid *g, double dt0, double dt1, double threshold, int *launches)
+{
+    PrologueArgs a;
+    a.dt[0] = dt0;
+    a.dt[1] = dt1;
+    a.threshold = threshold;
+    for (int i = 0; i < 2; ++i) a.build[i] = a.dt[i] != g->up_dt[i];
+    if (!a.build[0] && !a.build[1] && threshold == 0.0) return HJ_OK;
+    const bool tables = g->prec != HJ_FP32;
+    const int entries = g->n[2] * g->p4;
+    const int blocks = !tables ? 1 : (entries + 255) / 256 < 64 ? (entries + 255) / 256 : 64;
+    prologue_kernel<<<blocks, 256, 0, g->stream>>>(g->loop, a, g->geom,
+                                                   tables ? (const HjCoef<double> *)g->coef : nullptr, g->scaled,
+                                                   g->qw, tables ? (const double *)g->k4tab : nullptr);
+    HJ_CUDA(cudaGetLastError());
+    g->up_dt[0] = dt0;
+    g->up_dt[1] = dt1;
+    ++*launches;
+    return HJ_OK;
 }
 
 void free_grid(hj_grid *g)
@@ -431,14 +465,14 @@ void free_grid(hj_grid *g)
     if (g->buf) cudaFree(g->buf);
     if (g->coef) cudaFree(g->coef);
     if (g->tab_tiled) cudaFree(g->tab_tiled);
-    if (g->amax_q) cudaFree(g->amax_q);
     if (g->scaled) cudaFree(g->scaled);
     if (g->qw) cudaFree(g->qw);
     if (g->v0xy) cudaFree(g->v0xy);
     if (g->k4tab) cudaFree(g->k4tab);
     if (g->rsync) cudaFree(g->rsync);
-    if (g->dstate) cudaFree(g->dstate);
-    if (g->hstate) cudaFreeHost(g->hstate);
+    if (g->loop) cudaFree(g->loop);
+    if (g->hloop) cudaFreeHost(g->hloop);
+    if (g->hflags) cudaFreeHost(g->hflags);
     for (int i = 0; i < 4; ++i)
         if (g->ev[i]) cudaEventDestroy(g->ev[i]);
     if (g->ev_in) cudaEventDestroy(g->ev_in);
@@ -487,7 +521,7 @@ cudaError_t hj_launch_readback_f32(const float *src, void *dst, hj_precision dst
 cudaError_t hj_launch_prologue_f32(HjDevState *st, const HjGeom &g, const HjCoef<float> *coef, int ncoef, double T,
                                    double cfl, cudaStream_t stream)
 {
-    prologue_kernel<float><<<1, 256, 0, stream>>>(st, g, coef, ncoef, T, cfl);
+    slot_prologue_kernel<<<1, 256, 0, stream>>>(st, g, coef, ncoef, T, cfl);
     return cudaGetLastError();
 }
 
@@ -562,18 +596,20 @@ hj_status hj_create_grid(const int32_t n[4], const double lo[4], const double hi
     if (e == cudaSuccess) e = cudaMalloc(&g->buf, 2 * arr);
     // FP64 coefficients for FP64 and Q5.27 grids (alpha^max and dt are FP64)
     const size_t coef_bytes = ncoef * (prec == HJ_FP32 ? sizeof(HjCoef<float>) : sizeof(HjCoef<double>));
-    const size_t qw_bytes = prec == HJ_Q527 ? sizeof(int32_t) * (2 * (size_t)n[2] * g->p4 + HJ_QW_TAIL + n[2]) : 0;
+    const size_t qw_bytes = prec == HJ_Q527 ? 2 * sizeof(int32_t) * hj_qw_count(n[2], g->p4) : 0;
+    const size_t scaled_bytes = prec == HJ_FP64 ? 2 * ncoef * sizeof(HjScaledCoef) : 0;
     const size_t k4_bytes = (size_t)n[2] * (prec == HJ_FP32 ? 2 * sizeof(float) : sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&g->coef, coef_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&g->tab_tiled, sizeof(float) * ((size_t)n[2] + 3 * (size_t)g->p4));
-    if (e == cudaSuccess) e = cudaMalloc(&g->amax_q, sizeof(double2) * (size_t)n[2] * (g->p4 / 4));
-    if (e == cudaSuccess && prec == HJ_FP64) e = cudaMalloc(&g->scaled, ncoef * sizeof(HjScaledCoef));
+    if (e == cudaSuccess && prec == HJ_FP64) e = cudaMalloc(&g->scaled, scaled_bytes);
     if (e == cudaSuccess && prec == HJ_Q527) e = cudaMalloc(&g->qw, qw_bytes);
     const size_t xy_bytes = (size_t)n[0] * n[1] * g->esize;
     if (e == cudaSuccess) e = cudaMalloc(&g->v0xy, xy_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&g->k4tab, k4_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&g->dstate, sizeof(HjDevState));
-    if (e == cudaSuccess) e = cudaHostAlloc(&g->hstate, sizeof(HjDevState), cudaHostAllocDefault);
+    if (e == cudaSuccess) e = cudaMalloc(&g->loop, sizeof(HjLoop));
+    if (e == cudaSuccess) e = cudaHostAlloc(&g->hloop, sizeof(HjLoop), cudaHostAllocDefault);
+    if (e == cudaSuccess) e = cudaHostAlloc(&g->hflags, sizeof(HjFlags), cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&g->dflags, g->hflags, 0);
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&g->ev[i]);
     if (e == cudaSuccess && g->own_stream) e = cudaEventCreateWithFlags(&g->ev_in, cudaEventDisableTiming);
     if (e != cudaSuccess) {
@@ -583,17 +619,8 @@ hj_status hj_create_grid(const int32_t n[4], const double lo[4], const double hi
         free_grid(g);
         return s;
     }
-    g->device_bytes = 3 * arr + coef_bytes + qw_bytes + (prec == HJ_FP64 ? ncoef * sizeof(HjScaledCoef) : 0) +
-                      xy_bytes + k4_bytes + sizeof(HjDevState);
-    hj_status s = reset_state(g);
-    if (s == HJ_OK) {
-        cudaError_t e2 = cudaStreamSynchronize(g->stream);
-        if (e2 != cudaSuccess) s = set_err(HJ_ERR_CUDA, "hj_create_grid: %s", cudaGetErrorString(e2));
-    }
-    if (s != HJ_OK) {
-        free_grid(g);
-        return s;
-    }
+    g->device_bytes = 3 * arr + coef_bytes + qw_bytes + scaled_bytes + xy_bytes + k4_bytes + sizeof(HjLoop);
+    reset_state(g);
     *out = g;
     return HJ_OK;
 }
@@ -663,11 +690,10 @@ hj_status hj_set_dynamics(hj_grid *g, hj_dynamics kind, const double *params, in
     G.k3 = G.alpha3 / g->h[2];
     G.k4 = G.alpha4 / g->h[3];
     if ((s = upload_tables(g)) != HJ_OK) return s;
-    // a solve in progress continues under the new dynamics: the next
-    // prologue re-reduces alpha^max from the new table (Alg. 2 takes it from
-    // the current Hamiltonian) and rebuilds the FP64 dt-scaled table
-    HJ_CUDA(cudaMemsetAsync(&g->dstate->dt_scaled, 0, sizeof(double), g->stream));
-    HJ_CUDA(cudaMemsetAsync(&g->dstate->alpha_stale, 1, sizeof(int), g->stream));
+    // a solve in progress continues under the new dynamics, with alpha^max of
+    // the new table (Alg. 2 takes it from the current Hamiltonian); the next
+    // prologue rebuilds the dt-scaled tables
+    g->up_dt[0] = g->up_dt[1] = -1.0;
     g->has_dyn = true;
     char why[160];
     g->tiled_ok = hj_tiled_setup(g, why, sizeof(why));
@@ -696,7 +722,7 @@ static hj_status finish_ingest(hj_grid *g);
 // broadcast-V0 step kernel, with the same conversion.
 static hj_status ingest_xy(hj_grid *g, const void *src, hj_precision dtype, long long nxy)
 {
-    int *flag = &g->dstate->nonfinite;
+    int *flag = &g->dflags->nonfinite;
     const int blocks = grid_blocks(g->nint, 256);
     with_elem(dtype, [&](auto ein) {
         with_elem(g->prec, [&](auto e) {
@@ -716,11 +742,9 @@ static hj_status finish_ingest(hj_grid *g)
 {
     HJ_CUDA(cudaGetLastError());
     HJ_CUDA(cudaStreamSynchronize(g->stream));
-    HJ_CUDA(cudaMemcpy(g->hstate, g->dstate, sizeof(HjDevState), cudaMemcpyDeviceToHost));
-    if (g->hstate->nonfinite) {
+    if (*(volatile int *)&g->hflags->nonfinite) {
         g->has_value = false;
         reset_state(g);
-        cudaStreamSynchronize(g->stream);
         return set_err(HJ_ERR_INVALID_ARG, "V0 contains NaN or Inf");
     }
     g->has_value = true;
@@ -763,7 +787,7 @@ hj_status hj_set_initial_value(hj_grid *g, const double *v0, size_t count)
     if (count != (size_t)g->ncell)
         return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2*N3*N4 = %lld", count, g->ncell);
     if ((s = activate(g)) != HJ_OK) return s;
-    if ((s = reset_state(g)) != HJ_OK) return s;
+    reset_state(g);
     // pinned host memory: the ingest kernel reads it directly; otherwise stage
     // the dense FP64 array in the ping-pong region (2 * nint * esize >= ncell * 8 bytes)
     const double *staging = (const double *)device_view(g, v0);
@@ -772,7 +796,7 @@ hj_status hj_set_initial_value(hj_grid *g, const double *v0, size_t count)
         HJ_CUDA(cudaMemcpyAsync(g->buf, v0, sizeof(double) * (size_t)g->ncell, cudaMemcpyHostToDevice, g->stream));
     }
     long long nrows = (long long)g->n[0] * g->n[1] * g->n[2];
-    int *flag = &g->dstate->nonfinite;
+    int *flag = &g->dflags->nonfinite;
     int blocks = grid_blocks(g->nint, 256);
     with_elem(g->prec, [&](auto e) {
         using T = decltype(e);
@@ -791,7 +815,7 @@ hj_status hj_set_initial_value_xy(hj_grid *g, const double *v0_xy, size_t count)
     const long long nxy = (long long)g->n[0] * g->n[1];
     if (count != (size_t)nxy) return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2 = %lld", count, nxy);
     if ((s = activate(g)) != HJ_OK) return s;
-    if ((s = reset_state(g)) != HJ_OK) return s;
+    reset_state(g);
     double *staging = (double *)g->buf;  // N1*N2 doubles fit in the ping-pong region
     HJ_CUDA(cudaMemcpyAsync(staging, v0_xy, sizeof(double) * (size_t)nxy, cudaMemcpyHostToDevice, g->stream));
     return ingest_xy(g, staging, HJ_FP64, nxy);
@@ -808,7 +832,7 @@ hj_status hj_set_initial_value_xy_device(hj_grid *g, const void *v0_xy_device, h
     if (count != (size_t)nxy) return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2 = %lld", count, nxy);
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;
-    if ((s = reset_state(g)) != HJ_OK) return s;
+    reset_state(g);
     return ingest_xy(g, v0_xy_device, dtype, nxy);
 }
 
@@ -823,9 +847,9 @@ hj_status hj_set_initial_value_device(hj_grid *g, const void *v0_device, hj_prec
         return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2*N3*N4 = %lld", count, g->ncell);
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;
-    if ((s = reset_state(g)) != HJ_OK) return s;
+    reset_state(g);
     long long nrows = (long long)g->n[0] * g->n[1] * g->n[2];
-    int *flag = &g->dstate->nonfinite;
+    int *flag = &g->dflags->nonfinite;
     int blocks = grid_blocks(g->nint, 256);
     with_elem(dtype, [&](auto ein) {
         with_elem(g->prec, [&](auto e) {
@@ -867,60 +891,82 @@ static hj_status advance_loop(hj_grid *g, double T, double cfl, int64_t max_step
 
     const hj_kernel kern = effective_kernel(g);
     int launches = 0;
+    double dt = 0.0;
+    if (read_status(g) == HJ_OK && g->t < T && !cfl_step(g, cfl, &dt)) g->hflags->status = HJ_ERR_UNSTABLE;
+    if (read_status(g) != HJ_OK)
+        return set_err((hj_status)read_status(g), "device reported %s", hj_status_string((hj_status)read_status(g)));
     HJ_CUDA(cudaEventRecord(g->ev[0], g->stream));
-    launch_prologue(g, T, cfl, threshold);
-    ++launches;
-    HJ_CUDA(cudaGetLastError());
-    if ((s = pull_state(g)) != HJ_OK) return s;
-    const long long n_start = g->hstate->n;
-    const double dt_first = g->hstate->done ? 0.0 : g->hstate->dt;
-    long long taken = 0;
-    bool loop_started = false;
-    while (!g->hstate->done && g->hstate->status == HJ_OK && taken < max_steps) {
-        // predicted steps to the horizon (dt is constant until the cut last step)
-        const HjDevState &h = *g->hstate;
-        long long k = 1;
-        if (!h.last && h.dt > 0) {
-            double r = ceil((h.T - h.t) / h.dt);
-            k = r > 1 ? (r < 1e15 ? (long long)r : (long long)1e15) : 1;
+    const long long n_start = g->nstep;
+    double t = g->t, dt_first = 0.0, dt_last = 0.0, last_change = 0.0;
+    bool loop_started = false, converged = false;
+    // the resident kernel ends a converging loop itself; the others' steps
+    // are queued 32 at a time and the test's outcome is read in between
+    const long long chunk_max = threshold > 0.0 && kern != HJ_KERNEL_RESIDENT ? 32 : 1 << 16;
+    while (t < T && !converged && g->nstep - n_start < max_steps) {
+        // the next steps: dt each, and the one that reaches T cut to land on it
+        long long left = max_steps - (g->nstep - n_start), k = 0;
+        if (left > chunk_max) left = chunk_max;
+        double te = t, dt_cut = g->up_dt[1];
+        bool cut = false;
+        while (te < T && k < left) {
+            cut = dt == 0.0 || te + dt >= T;
+            if (cut) dt_cut = T - te;
+            te = cut ? T : te + dt;
+            ++k;
         }
-        if (k > max_steps - taken) k = max_steps - taken;
-        // the resident kernel ends the loop itself (horizon, convergence)
-        if (kern == HJ_KERNEL_RESIDENT) k = max_steps - taken;
-        if (threshold > 0.0 && k > 32 && kern != HJ_KERNEL_RESIDENT) k = 32;  // graphs: look every 32 steps
-        if (k > (1 << 16)) k = 1 << 16;  // read the device state (and any error) at least this often
+        if ((s = launch_prologue(g, dt, dt_cut, threshold, &launches)) != HJ_OK) return s;
         if (!loop_started) {
             HJ_CUDA(cudaEventRecord(g->ev[1], g->stream));
             loop_started = true;
         }
         if (kern == HJ_KERNEL_RESIDENT) {
-            HJ_CUDA(hj_launch_step_resident(g, k));
+            HJ_CUDA(hj_launch_step_resident(g, g->nstep, k, cut));
             ++launches;
-        } else if (launch_steps_graph(g, kern, k)) {
+        } else if (launch_steps_graph(g, kern, g->nstep, k, cut)) {
             launches += (int)k;
         } else {
             for (long long i = 0; i < k; ++i) {
-                if ((s = launch_step(g, kern)) != HJ_OK) return s;
+                if ((s = launch_step(g, kern, g->nstep + i, cut && i == k - 1)) != HJ_OK) return s;
                 ++launches;
             }
         }
         HJ_CUDA(cudaEventRecord(g->ev[2], g->stream));
-        if ((s = pull_state(g)) != HJ_OK) return s;
-        taken = g->hstate->n - n_start;
+        long long taken = k;
+        if (threshold > 0.0) {
+            HJ_CUDA(cudaMemcpyAsync(g->hloop, g->loop, sizeof(HjLoop), cudaMemcpyDeviceToHost, g->stream));
+            HJ_CUDA(cudaEventRecord(g->ev[3], g->stream));
+            if ((s = wait_stream(g)) != HJ_OK) return s;
+            taken = g->hloop->taken;
+            last_change = g->hloop->delta_last;
+            converged = g->hloop->done != 0;
+        } else {
+            HJ_CUDA(cudaEventRecord(g->ev[3], g->stream));
+            if ((s = wait_stream(g)) != HJ_OK) return s;
+        }
+        // a timed-out wait: the values are not those of any step
+        if (read_status(g) != HJ_OK)
+            return set_err((hj_status)read_status(g), "device reported %s",
+                           hj_status_string((hj_status)read_status(g)));
+        for (long long i = 0; i < taken; ++i) {
+            dt_last = cut && i == k - 1 ? dt_cut : dt;
+            if (dt_first == 0.0) dt_first = dt_last;
+            t = cut && i == k - 1 ? T : t + dt;
+        }
+        g->t = t;
+        g->nstep += taken;
     }
-    HJ_CUDA(cudaEventRecord(g->ev[3], g->stream));
-    HJ_CUDA(cudaEventSynchronize(g->ev[3]));
-    const HjDevState &h = *g->hstate;
-    if (h.status != HJ_OK)
-        return set_err((hj_status)h.status, "device reported %s", hj_status_string((hj_status)h.status));
+    if (!loop_started) {
+        HJ_CUDA(cudaEventRecord(g->ev[3], g->stream));
+        HJ_CUDA(cudaEventSynchronize(g->ev[3]));
+    }
     if (stats) {
         memset(stats, 0, sizeof(*stats));
-        stats->steps = h.n - n_start;
-        stats->total_steps = h.n;
-        stats->t_final = h.t;
-        stats->dt_first = stats->steps > 0 ? dt_first : 0.0;
-        stats->dt_last = stats->steps > 0 ? h.dt_prev : 0.0;
-        for (int d = 0; d < 4; ++d) stats->alpha_max[d] = h.alpha_prev[d];
+        stats->steps = g->nstep - n_start;
+        stats->total_steps = g->nstep;
+        stats->t_final = g->t;
+        stats->dt_first = dt_first;
+        stats->dt_last = dt_last;
+        for (int d = 0; d < 4; ++d) stats->alpha_max[d] = g->alpha[d];
         float ms = 0.f;
         cudaEventElapsedTime(&ms, g->ev[0], g->ev[3]);
         stats->device_ms = ms;
@@ -930,8 +976,8 @@ static hj_status advance_loop(hj_grid *g, double T, double cfl, int64_t max_step
         }
         stats->kernel = kern;
         stats->launches = launches;
-        stats->last_change = h.delta_last;
-        stats->converged = h.converged;
+        stats->last_change = last_change;
+        stats->converged = converged ? 1 : 0;
     }
     return HJ_OK;
 }
@@ -970,8 +1016,7 @@ hj_status hj_read_value(const hj_grid *gc, double *out, size_t count)
         return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2*N3*N4 = %lld", count, g->ncell);
     if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
     if ((s = activate(g)) != HJ_OK) return s;
-    if ((s = pull_state(g)) != HJ_OK) return s;
-    const long long n = g->hstate->n;
+    const long long n = g->nstep;
     const void *src = hj_value_ptr(g, n);
     const long long nrows = (long long)g->n[0] * g->n[1] * g->n[2];
     // pinned host memory: the readback kernel writes it directly, in one pass
@@ -1031,8 +1076,7 @@ hj_status hj_query_device(const hj_grid *gc, const double *states, int64_t m, do
     if (control && !g->has_dyn) return set_err(HJ_ERR_STATE, "the control needs the dynamics (hj_set_dynamics)");
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;
-    if ((s = pull_state(g)) != HJ_OK) return s;
-    HJ_CUDA(hj_launch_query(g, hj_value_ptr(g, g->hstate->n), states, m, value, grad, control));
+    HJ_CUDA(hj_launch_query(g, hj_value_ptr(g, g->nstep), states, m, value, grad, control));
     HJ_CUDA(cudaStreamSynchronize(g->stream));
     return HJ_OK;
 }
@@ -1048,8 +1092,7 @@ hj_status hj_query(const hj_grid *gc, const double *states, int64_t m, double *v
     if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
     if (control && !g->has_dyn) return set_err(HJ_ERR_STATE, "the control needs the dynamics (hj_set_dynamics)");
     if ((s = activate(g)) != HJ_OK) return s;
-    if ((s = pull_state(g)) != HJ_OK) return s;
-    const long long n = g->hstate->n;
+    const long long n = g->nstep;
     // stage states and results in the buffer the next step writes (free now)
     char *free_buf;
     size_t free_bytes;
@@ -1093,8 +1136,7 @@ hj_status hj_read_value_device(const hj_grid *gc, void *out_device, hj_precision
     if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;  // the output array too
-    if ((s = pull_state(g)) != HJ_OK) return s;
-    const void *src = hj_value_ptr(g, g->hstate->n);
+    const void *src = hj_value_ptr(g, g->nstep);
     const long long nrows = (long long)g->n[0] * g->n[1] * g->n[2];
     int blocks = grid_blocks(g->ncell, 256);
     with_elem(g->prec, [&](auto e) {
@@ -1161,9 +1203,9 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
     if (!g->tiled_ok) return set_err(HJ_ERR_UNSUPPORTED, "this grid has no tiled kernel");
     if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
     if ((s = activate(g)) != HJ_OK) return s;
-    if ((s = pull_state(g)) != HJ_OK) return s;
-    if (g->hstate->n != 0) return set_err(HJ_ERR_STATE, "autotune must run before the first step");
-    HjDevState saved = *g->hstate;
+    if (g->nstep != 0) return set_err(HJ_ERR_STATE, "autotune must run before the first step");
+    double dt_trial = 0.0;
+    if (!cfl_step(g, 0.8, &dt_trial)) return set_err(HJ_ERR_UNSTABLE, "the CFL step is not a usable number");
     int32_t keep[4];
     memcpy(keep, g->tile_req, sizeof(keep));
 
@@ -1203,16 +1245,15 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
     // CTAs (the only candidate on a grid too small for the classes above)
     cands[nc++] = {0, 0, 0.0};
 
+    // k steps from V0 (the trials leave t and the step count at 0, so nothing
+    // has to be put back)
+    int launches = 0;
     auto run_steps = [&](int k) -> hj_status {
-        *g->hstate = saved;
-        HJ_CUDA(cudaMemcpyAsync(g->dstate, g->hstate, sizeof(HjDevState), cudaMemcpyHostToDevice, g->stream));
-        launch_prologue(g, 1e300, 0.8);
-        HJ_CUDA(cudaGetLastError());
+        hj_status r = launch_prologue(g, dt_trial, g->up_dt[1], 0.0, &launches);
+        if (r != HJ_OK) return r;
         HJ_CUDA(cudaEventRecord(g->ev[1], g->stream));
-        for (int i = 0; i < k; ++i) {
-            hj_status r = launch_step(g, HJ_KERNEL_TILED);
-            if (r != HJ_OK) return r;
-        }
+        for (int i = 0; i < k; ++i)
+            if ((r = launch_step(g, HJ_KERNEL_TILED, i, 0)) != HJ_OK) return r;
         HJ_CUDA(cudaEventRecord(g->ev[2], g->stream));
         HJ_CUDA(cudaEventSynchronize(g->ev[2]));
         return HJ_OK;
@@ -1233,10 +1274,9 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
             else if (g->tile_xc == auto_xc) continue;  // the automatic choice already was one chunk
             if ((s = run_steps(2)) != HJ_OK) break;  // warm-up
             if ((s = run_steps(steps_per_trial)) != HJ_OK) break;
-            pull_state(g);
-            if (g->hstate->status != HJ_OK) {
-                s = set_err((hj_status)g->hstate->status, "device reported %s during autotune",
-                            hj_status_string((hj_status)g->hstate->status));
+            if (read_status(g) != HJ_OK) {
+                s = set_err((hj_status)read_status(g), "device reported %s during autotune",
+                            hj_status_string((hj_status)read_status(g)));
                 break;
             }
             float ms = 0.f;
@@ -1293,7 +1333,7 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
             }
         }
     }
-    // keep the winner (or the previous shape if nothing ran), restore the state
+    // keep the winner (or the previous shape if nothing ran)
     if (best < 1e300)
         memcpy(g->tile_req, best_req, sizeof(best_req));
     else
@@ -1306,9 +1346,6 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
               g->tile_stages != best_req[3]))
         s = set_err(HJ_ERR_CUDA, "autotune: tile shape (%d, %d, %d, %d) came out as (%d, %d, %d, %d)", best_req[0],
                     best_req[1], best_req[2], best_req[3], g->tile_ty, g->tile_tv, g->tile_xc, g->tile_stages);
-    *g->hstate = saved;
-    cudaMemcpyAsync(g->dstate, g->hstate, sizeof(HjDevState), cudaMemcpyHostToDevice, g->stream);
-    cudaStreamSynchronize(g->stream);
     if (nresults) *nresults = count;
     return s;
 }
@@ -1319,8 +1356,6 @@ hj_status hj_get_info(const hj_grid *g, hj_grid_info *info)
     hj_status s = check_grid(g);
     if (s != HJ_OK) return s;
     if (!info) return set_err(HJ_ERR_INVALID_ARG, "info is NULL");
-    if ((s = activate(g)) != HJ_OK) return s;
-    if ((s = pull_state((hj_grid *)g)) != HJ_OK) return s;
     memset(info, 0, sizeof(*info));
     for (int d = 0; d < 4; ++d) {
         info->n[d] = g->n[d];
@@ -1334,8 +1369,8 @@ hj_status hj_get_info(const hj_grid *g, hj_grid_info *info)
     info->kernel = effective_kernel(g);
     info->periodic_mask = g->periodic;
     info->has_value = g->has_value;
-    info->total_steps = g->hstate->n;
-    info->t = g->hstate->t;
+    info->total_steps = g->nstep;
+    info->t = g->t;
     info->device_bytes = g->device_bytes;
     if (g->tiled_ok) {
         info->tile[0] = g->tile_ty;

@@ -139,7 +139,7 @@ __global__ void batch_horizon_many_kernel(const SlotSetup *__restrict__ list)
 {
     __shared__ unsigned long long scratch[64];
     const SlotSetup &d = list[blockIdx.x];
-    hj_prologue_block(d.st, d.geom, d.coef, d.ncoef, d.T, d.cfl, 0.0, scratch);
+    hj_prologue_block(d.st, d.geom, d.coef, d.ncoef, d.T, d.cfl, scratch);
 }
 
 // What the consumers need of a work item, written into shared memory by the

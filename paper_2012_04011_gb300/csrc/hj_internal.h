@@ -16,9 +16,9 @@ enum HjAxisMode : int32_t {
     HJ_AXIS_MINUS = 2     // fixed velocity < 0: upwind value is V-
 };
 
-// Device-resident time-loop state of one grid.  Written by the prologue
-// kernel and by the last CTA of every step kernel ("finaliser"), read by the
-// next kernel on the same stream.
+// Device-resident time-loop state of one batch slot.  Written by the
+// prologue kernels and by the warp that finalises the slot's step, read by
+// the slot's next step.
 struct HjDevState {
     double t;                          // simulated time at the start of the next step
     double dt;                         // size of the next step
@@ -27,19 +27,35 @@ struct HjDevState {
     double cfl;                        // Courant number of the current call
     long long n;                       // steps since V0 was set
     int last;                          // the next step is cut to land on T
-    int done;                          // t has reached T: step kernels exit at once
+    int done;                          // t has reached T
     unsigned long long alpha_bits[2];  // running max of |xdot_1|, |xdot_2| of this step (FP64 bit patterns)
     double alpha_prev[4];              // alpha_d^max reduced by the last step (or the prologue)
-    unsigned int blocks_done;          // CTAs of the current step that have finished
     int status;                        // hj_status raised on the device (HJ_OK if none)
     int nonfinite;                     // ingest saw a NaN or Inf
-    int alpha_stale;                   // dynamics changed: the next prologue re-reduces alpha^max
-    double dt_scaled;                  // dt the FP64 dt-scaled coefficient table holds (0: none yet)
-    int track;                         // convergence mode: the steps reduce max |V_{n+1} - V_n|
-    int converged;                     // the last step changed V by less than the threshold
-    double threshold;                  // convergence threshold of the current call
-    unsigned long long delta_bits;     // running max |V_{n+1} - V_n| of this step (FP64 bit pattern)
-    double delta_last;                 // max |V_{n+1} - V_n| of the step just taken (convergence mode)
+};
+
+// Device constants of a grid's current solve call, written by its prologue
+// kernel.  alpha^max of every supported dynamics is a property of the (v,
+// theta) tables and not of V, so the host runs Algorithm 1's time loop (same
+// FP64 operations as the oracle) and a step kernel only needs the step size:
+// dt[0], or dt[1] for the step that is cut to land on the horizon.  The rest
+// is the convergence mode's state.
+struct HjLoop {
+    double dt[2];
+    double threshold;               // convergence threshold
+    double delta_last;              // max |V_{n+1} - V_n| of the step just taken
+    unsigned long long delta_bits;  // its running maximum (FP64 bit pattern)
+    long long taken;                // steps taken since the prologue
+    int done;                       // converged: later steps exit at once
+    unsigned int blocks_done;       // CTAs of the current step that have finished
+};
+
+// Host-visible flags of a grid (pinned host memory mapped into the device):
+// kernels store here only when something is wrong, and the host reads them
+// after the synchronisation that ends a call, without a copy of its own.
+struct HjFlags {
+    int status;     // hj_status raised on the device (HJ_OK if none)
+    int nonfinite;  // an ingest saw a NaN or Inf
 };
 
 // FP64 coefficients with dt folded in (per (v, theta)): w1 = dt xdot_1/dx_1,
@@ -98,18 +114,24 @@ struct hj_grid {
     void *v0;              // V0 (internal layout)
     void *buf;             // two ping-pong buffers, back to back (2*nint values)
     void *coef;            // HjCoef<T>[n3*n4]
-    HjScaledCoef *scaled;  // FP64 grids: dt-scaled coefficients [n3*n4]
-    int32_t *qw;           // Q5.27 grids: fixed-point axis weights (hj_rescale_qweights)
+    HjScaledCoef *scaled;  // FP64 grids: dt-scaled coefficients [n3*n4], one table per entry of HjLoop::dt
+    int32_t *qw;           // Q5.27 grids: fixed-point axis weights (hj_rescale_qweights), likewise two tables
     void *k4tab;           // theta coefficient per speed: |xdot_4|/dx_4 (double[n3]; FP32 grids: float2[n3] of
                            // (k4, -(k3 + k4)))
     void *v0xy;            // V0 as an N1 x N2 field (element type of the grid), when V0 depends on x, y only
     bool v0_bcast;         // V0 was set from the (x, y) field: the tiled kernel reads v0xy
     bool track;            // a convergence-mode call is running: launch the kernels that reduce the change
     float *tab_tiled;      // tiled-kernel tables: v_k [n3], cos/dx1 [p4], sin/dx2 [p4], quad signs [p4]
-    double2 *amax_q;       // per (v_k, theta quad q) [n3][p4 / 4]: the largest FP64 |xdot_1|, |xdot_2| over the
-                           // quad's headings (the tiled kernel's alpha^max partials, one load per work item)
-    HjDevState *dstate;
-    HjDevState *hstate;    // pinned host mirror
+    HjLoop *loop;          // device constants of the current solve call
+    HjLoop *hloop;         // pinned host copy (convergence mode)
+    HjFlags *hflags;       // pinned, mapped
+    HjFlags *dflags;       // its device address
+
+    // the time loop's state: Algorithm 1 runs on the host
+    double t;              // simulated time
+    long long nstep;       // steps since V0 was set
+    double alpha[4];       // alpha_d^max of the current dynamics (over the grid's (v, theta) states)
+    double up_dt[2];       // step sizes the device constants and dt-scaled tables hold (0: none)
 
     bool has_dyn, has_value;
     hj_dynamics dyn;
@@ -130,7 +152,7 @@ struct hj_grid {
     // value, so a graph is valid while `launch_version` is unchanged
     struct StepGraph {
         long long k;
-        int kernel, track;
+        int kernel, track, cut, parity;  // parity: which buffers the first step reads and writes
         unsigned version;
         cudaGraphExec_t exec;
     } graphs[4];
@@ -140,12 +162,14 @@ struct hj_grid {
     size_t device_bytes;
 };
 
-// Launchers (each returns the CUDA error of its launch).
-cudaError_t hj_launch_step_generic(hj_grid *g);
-cudaError_t hj_launch_step_tiled(hj_grid *g);
-// Up to k steps in one cooperative launch of the resident kernel (it stops
-// early when the time loop is done); allocates g->rsync on first use.
-cudaError_t hj_launch_step_resident(hj_grid *g, long long k);
+// Launchers of one step, from V after n steps with step size dt[sel] (each
+// returns the CUDA error of its launch).
+cudaError_t hj_launch_step_generic(hj_grid *g, long long n, int sel);
+cudaError_t hj_launch_step_tiled(hj_grid *g, long long n, int sel);
+// k steps from V after n steps in one cooperative launch of the resident
+// kernel, the last of them with dt[1] if cut (convergence mode: it stops early
+// when the test ends the loop); allocates g->rsync on first use.
+cudaError_t hj_launch_step_resident(hj_grid *g, long long n, long long k, bool cut);
 // Whether the device can run the resident kernel (cooperative launch).
 bool hj_resident_supported(const hj_grid *g);
 // Set up the tiled kernel for g (tensor maps, tile shape); false if unsupported.
@@ -183,11 +207,8 @@ cudaError_t hj_launch_readback_f32(const float *src, void *dst, hj_precision dst
 cudaError_t hj_launch_prologue_f32(HjDevState *st, const HjGeom &g, const HjCoef<float> *coef, int ncoef, double T,
                                    double cfl, cudaStream_t stream);
 
-// Rescale the FP64 coefficient table for dt (all threads of one block call
-// it; the table covers n3 * n4 entries; k4 holds the theta coefficient of
-// each speed).
-// One entry of that table: coefficients c of a (v, theta), theta
-// coefficient k4 of the speed.
+// One entry of the FP64 dt-scaled table: coefficients c of a (v, theta),
+// theta coefficient k4 of the speed.
 __device__ __forceinline__ HjScaledCoef hj_scaled_entry(const HjCoef<double> &c, double k4, double dt)
 {
     HjScaledCoef o;
@@ -198,10 +219,12 @@ __device__ __forceinline__ HjScaledCoef hj_scaled_entry(const HjCoef<double> &c,
     return o;
 }
 
+// The table for dt, n3 * n4 entries, by `stride` threads of which the caller
+// is number `first` (k4: the theta coefficient of each speed).
 __device__ __forceinline__ void hj_rescale_table(HjScaledCoef *sc, const HjCoef<double> *coef, const double *k4,
-                                                 int n3, int n4, double dt)
+                                                 int n3, int n4, double dt, int first, int stride)
 {
-    for (int i = threadIdx.x; i < n3 * n4; i += blockDim.x) sc[i] = hj_scaled_entry(coef[i], k4[i / n4], dt);
+    for (int i = first; i < n3 * n4; i += stride) sc[i] = hj_scaled_entry(coef[i], k4[i / n4], dt);
 }
 
 // ---- Q5.27 fixed point (Sec. III-C, Sec. IV-B): int32 codes q, value q 2^-27
@@ -226,18 +249,25 @@ __device__ __forceinline__ int32_t hj_qweight(double dt, double k)
     return (int32_t)__double2ll_rn(__dmul_rn(__dmul_rn(dt, k), HJ_QW_SCALE));
 }
 
-// Fixed-point weights for dt (all threads of one block call it):
+// Fixed-point weights for dt (by `stride` threads of which the caller is
+// number `first`):
 //   qw[k p4 + l]            x weight of (v_k, theta_l), signed with xdot_1
 //   qw[n3 p4 + k p4 + l]    y weight, signed with xdot_2
 //   qw[2 n3 p4]             v weight (constant over the grid)
 //   qw[2 n3 p4 + 4 + k]     theta weight of speed v_k
 // Pad lanes (l >= n4) get 0.
 constexpr int HJ_QW_TAIL = 4;  // entries between the y weights and the per-speed theta weights
+// Entries of one such table, rounded up so that a second one behind it keeps
+// the rows' 16-byte alignment.
+__host__ __device__ __forceinline__ size_t hj_qw_count(int n3, int p4)
+{
+    return (2 * (size_t)n3 * p4 + HJ_QW_TAIL + n3 + 3) / 4 * 4;
+}
 __device__ __forceinline__ void hj_rescale_qweights(int32_t *qw, const HjCoef<double> *coef, int n3, int n4, int p4,
-                                                    double k3, const double *k4, double dt)
+                                                    double k3, const double *k4, double dt, int first, int stride)
 {
     const int tot = n3 * p4;
-    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+    for (int i = first; i < tot; i += stride) {
         const int k = i / p4, l = i - (i / p4) * p4;
         int32_t w1 = 0, w2 = 0;
         if (l < n4) {
@@ -250,8 +280,8 @@ __device__ __forceinline__ void hj_rescale_qweights(int32_t *qw, const HjCoef<do
         qw[i] = w1;
         qw[tot + i] = w2;
     }
-    for (int k = threadIdx.x; k < n3; k += blockDim.x) qw[2 * tot + HJ_QW_TAIL + k] = hj_qweight(dt, k4[k]);
-    if (threadIdx.x == 0) {
+    for (int k = first; k < n3; k += stride) qw[2 * tot + HJ_QW_TAIL + k] = hj_qweight(dt, k4[k]);
+    if (first == 0) {
         qw[2 * tot] = hj_qweight(dt, k3);
         qw[2 * tot + 1] = 0;
     }
@@ -315,7 +345,8 @@ __device__ __forceinline__ int32_t hj_q527_update(int32_t vc, int32_t v0, long l
 hj_status hj_batch_refresh(hj_batch *b);
 bool hj_batch_cached_done(const hj_batch *b, int32_t slot, int64_t *steps);
 
-// Pointer of the value buffer that holds V after n steps.
+// Pointer of the value buffer that holds V after n steps (step n reads it and
+// writes hj_value_ptr(g, n + 1)).
 inline void *hj_value_ptr(const hj_grid *g, long long n)
 {
     if (n == 0) return g->v0;

@@ -49,7 +49,6 @@ __global__ void noalloc_init_kernel(HjDevState *st, HjCoef<T> *coef, const HjGeo
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->alpha_bits[0] = 0ull;
         st->alpha_bits[1] = 0ull;
-        st->blocks_done = 0u;
         st->status = HJ_OK;
     }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncoef; i += gridDim.x * blockDim.x) {

@@ -14,8 +14,7 @@
 // max(V+, V-).  Summing over axes:
 //     V_new = min(V0, V_c + dt * (sum_d K_d V_up,d - K_sum V_c)),
 // with K_d = |xdot_d| / dx_d.  The FP64 variant folds dt into a per-(v, theta)
-// table (w0 = 1 - dt K_sum, w_d = dt K_d): 1 DMUL + 4 DFMA per cell, the
-// table rescaled by the last CTA only when dt changes.  The FP32 variant
+// table (w0 = 1 - dt K_sum, w_d = dt K_d): 1 DMUL + 4 DFMA per cell.  The FP32 variant
 // keeps the differences (V_up - V_c) for accuracy.  The Q5.27 kernel
 // (hj_step_q527_kernel) evaluates the same form in exact integer differences
 // with fixed-point weights.
@@ -27,7 +26,6 @@
 #include <type_traits>
 
 #include "hj_resident.cuh"
-#include "hj_scaled.cuh"
 
 namespace {
 
@@ -136,10 +134,8 @@ __device__ __forceinline__ long long q_upwind(const QDiff &d, int mode)
 }
 
 // ---------------------------------------------------------- one cell's update
-// The resident kernel's FP32 / FP64 update and the Q5.27 update of both
-// forms.  hj_step_generic_kernel writes the same FP32 / FP64 expressions, in
-// the same order, inline (its FP64 build is 2 % faster that way), so the
-// resident and per-step kernels give the same result bit for bit (tested).
+// The updates of both the per-step and the resident kernels, which therefore
+// give the same result bit for bit (tested).
 
 // FP32: V_c + dt (K1 (V_up1 - V_c) + K2 (V_up2 - V_c) + k3 (V_up3 - V_c) +
 // k4 (V_up4 - V_c)), the Euler update before the BRT min with V0 (the caller
@@ -222,30 +218,19 @@ __device__ __forceinline__ Cell cell_at(unsigned long long c, const Divisors &dv
     return r;
 }
 
-// Per-thread maxima of a step: |xdot_1|, |xdot_2| and the change of V.
+// Per-thread largest change of V in a step (convergence mode).
 struct StepMax {
-    unsigned long long a1 = 0ull, a2 = 0ull, d = 0ull;  // FP64 bit patterns (Q5.27: d in codes)
-    float df = 0.f;                                     // FP32 kernels: the change of V
+    unsigned long long d = 0ull;  // FP64 bit pattern (Q5.27: codes)
+    float df = 0.f;               // FP32 kernels
 };
 
-// The maxima as bit patterns of non-negative doubles.
+// It as the bit pattern of a non-negative double.
 template <typename T>
-__device__ __forceinline__ void step_max_bits(const StepMax &m, unsigned long long &a1, unsigned long long &a2,
-                                              unsigned long long &d)
+__device__ __forceinline__ unsigned long long step_max_bits(const StepMax &m)
 {
-    if constexpr (std::is_same<T, float>::value) {
-        a1 = m.a1;
-        a2 = m.a2;
-        d = hj_abits((double)m.df);
-    } else if constexpr (std::is_same<T, double>::value) {
-        a1 = m.a1;
-        a2 = m.a2;
-        d = m.d;
-    } else {  // the largest change in codes, as the FP64 value it stands for (exact)
-        a1 = m.a1;
-        a2 = m.a2;
-        d = hj_abits((double)m.d * (1.0 / HJ_Q527_SCALE));
-    }
+    if constexpr (std::is_same<T, float>::value) return hj_abits((double)m.df);
+    else if constexpr (std::is_same<T, double>::value) return m.d;
+    else return hj_abits((double)m.d * (1.0 / HJ_Q527_SCALE));  // codes, as the FP64 value they stand for (exact)
 }
 
 // Largest change of V, per precision (convergence mode).
@@ -263,24 +248,19 @@ __device__ __forceinline__ void track_change(StepMax &m, int32_t vn, int32_t vc)
 }
 
 // One step in Q5.27 for every grid (the tiled kernel covers the car grids it
-// supports).  alpha^max comes from the FP64 table, so the dt sequence is the
-// FP64 one.
+// supports); qw holds the weights of this step's dt.
 template <bool FAST32, bool TRACK>
-__global__ void __launch_bounds__(256) hj_step_q527_kernel(const int32_t *__restrict__ v0, int32_t *__restrict__ buf,
-                                                            const HjCoef<double> *__restrict__ coef, int32_t *qw,
-                                                            const double *__restrict__ k4tab, HjDevState *st,
-                                                            const HjGeom g, long long nint, const Divisors dv)
+__global__ void __launch_bounds__(256) hj_step_q527_kernel(const int32_t *__restrict__ v0,
+                                                            const int32_t *__restrict__ vin, int32_t *__restrict__ vout,
+                                                            const int32_t *__restrict__ qw, HjLoop *lp, const HjGeom g,
+                                                            const Divisors dv)
 {
-    __shared__ unsigned long long scratch[96];
+    __shared__ unsigned long long scratch[32];
     // a programmatic dependent of the previous step: wait for its grid (its
-    // V_n and finalised state), then let the next step be scheduled
+    // V_n), then let the next step be scheduled
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (st->done) return;
+    if (TRACK && lp->done) return;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long n = st->n;
-    const int32_t *vin;
-    int32_t *vout;
-    hj_io_buffers<int32_t>(v0, buf, nint, n, vin, vout);
 
     const long long s2 = (long long)g.n3 * g.p4, s1 = (long long)g.n2 * s2;
     const unsigned long long ncell = (unsigned long long)g.n1 * g.n2 * g.n3 * g.n4;
@@ -301,34 +281,25 @@ __global__ void __launch_bounds__(256) hj_step_q527_kernel(const int32_t *__rest
                                         qw[tot + cl.k * g.p4 + cl.l], w3, w4tab[cl.k], g.mode3, g.mode4);
         vout[o] = vn;
         if constexpr (TRACK) track_change(m, vn, vc);  // convergence mode: largest change of V
-        const HjCoef<double> cf = coef[cl.k * g.n4 + cl.l];
-        const unsigned long long b1 = hj_abits(cf.a1), b2 = hj_abits(cf.a2);
-        m.a1 = m.a1 > b1 ? m.a1 : b1;
-        m.a2 = m.a2 > b2 ? m.a2 : b2;
     }
-    unsigned long long a1, a2, d;
-    step_max_bits<int32_t>(m, a1, a2, d);
-    hj_step_epilogue_scaled(st, g, a1, a2, d, scratch, nullptr, qw, coef, k4tab);
+    if constexpr (TRACK) hj_track_epilogue(lp, step_max_bits<int32_t>(m), scratch);
 }
 
 template <typename T, bool FAST32, bool TRACK>
-__global__ void __launch_bounds__(256) hj_step_generic_kernel(const T *__restrict__ v0, T *__restrict__ buf,
+__global__ void __launch_bounds__(256) hj_step_generic_kernel(const T *__restrict__ v0, const T *__restrict__ vin,
+                                                               T *__restrict__ vout,
                                                                const HjCoef<T> *__restrict__ coef,
-                                                               HjScaledCoef *scaled, const void *__restrict__ k4tab,
-                                                               HjDevState *st, const HjGeom g, long long nint,
-                                                               const Divisors dv)
+                                                               const HjScaledCoef *__restrict__ scaled,
+                                                               const void *__restrict__ k4tab, HjLoop *lp, int sel,
+                                                               const HjGeom g, const Divisors dv)
 {
-    __shared__ unsigned long long scratch[96];
+    __shared__ unsigned long long scratch[32];
     // a programmatic dependent of the previous step: wait for its grid (its
-    // V_n and finalised state), then let the next step be scheduled
+    // V_n), then let the next step be scheduled
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (st->done) return;  // uniform: written by the previous kernel on this stream
+    if (TRACK && lp->done) return;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long n = st->n;
-    const T dt = (T)st->dt;
-    const T *vin;
-    T *vout;
-    hj_io_buffers<T>(v0, buf, nint, n, vin, vout);
+    const T dt = (T)lp->dt[sel];
 
     const unsigned int N1 = g.n1, N2 = g.n2, N3 = g.n3, N4 = g.n4;
     const long long s3 = g.p4, s2 = (long long)N3 * g.p4, s1 = (long long)N2 * s2;
@@ -336,89 +307,57 @@ __global__ void __launch_bounds__(256) hj_step_generic_kernel(const T *__restric
     const T k3 = (T)g.k3;
     // FP64: dt is folded into the per-(v, theta) table; the v weight needs it
     // once per thread
-    const double k3dt = g.k3 * st->dt;
-    unsigned long long am1 = 0ull, am2 = 0ull, dbits = 0ull;
-    float dmf = 0.f;
+    const double k3dt = g.k3 * lp->dt[sel];
+    const bool per4 = (g.periodic >> 3) & 1, ctl = g.mode3 == HJ_AXIS_CONTROL && g.mode4 == HJ_AXIS_CONTROL;
+    StepMax mx;
 
     for (unsigned long long c = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; c < ncell;
          c += (unsigned long long)gridDim.x * blockDim.x) {
-        unsigned long long row;
-        int l, k, i, j;
-        if (FAST32) {  // the grid has fewer than 2^32 cells
-            const uint32_t c32 = (uint32_t)c, row32 = fast_div(c32, dv.n4);
-            const uint32_t r2 = fast_div(row32, dv.n3);
-            const uint32_t i32 = fast_div(r2, dv.n2);
-            row = row32;
-            l = (int)(c32 - row32 * N4);
-            k = (int)(row32 - r2 * N3);
-            i = (int)i32;
-            j = (int)(r2 - i32 * N2);
-        } else {
-            row = c / N4;
-            l = (int)(c - row * N4);
-            const unsigned long long r2 = row / N3;
-            k = (int)(row - r2 * N3);
-            i = (int)(r2 / N2);
-            j = (int)(r2 - (unsigned long long)i * N2);
-        }
-        const long long o = (long long)row * g.p4 + l;
+        const Cell cl = cell_at<FAST32>(c, dv, g);
+        const long long o = cl.o;
+        const int k = cl.k, l = cl.l;
 
         const T vc = vin[o];
-        const Neigh<T> nx = axis_neighbours<T>(vin, o, i, N1, s1, g.periodic & 1, vc);
-        const Neigh<T> ny = axis_neighbours<T>(vin, o, j, N2, s2, (g.periodic >> 1) & 1, vc);
-        const Neigh<T> nv = axis_neighbours<T>(vin, o, k, N3, s3, (g.periodic >> 2) & 1, vc);
-        const Neigh<T> nt = axis_neighbours<T>(vin, o, l, N4, 1, (g.periodic >> 3) & 1, vc);
-
-        const HjCoef<T> cf = coef[k * N4 + l];
-        const T u3 = upwind_value<T>(nv, g.mode3);
-        const T u4 = upwind_value<T>(nt, g.mode4);
         T vn;
         if constexpr (sizeof(T) == 8) {
-            // V_new = w0 V_c + |w1| V_up1 + |w2| V_up2 + dt k3 V_up3 + dt k4 V_up4:
-            // 1 DMUL + 4 DFMA; signs and magnitudes by integer operations
             const HjScaledCoef sc = scaled[k * N4 + l];
-            const T u1 = nonneg(sc.w1) ? nx.p : nx.m;
-            const T u2 = nonneg(sc.w2) ? ny.p : ny.m;
-            T r = sc.w0 * vc;
-            r = fma(mag(sc.w1), u1, r);
-            r = fma(mag(sc.w2), u2, r);
-            r = fma(k3dt, u3, r);
-            vn = fma(sc.w4, u4, r);
+            const bool inner = cl.i > 0 && cl.i < (int)N1 - 1 && cl.j > 0 && cl.j < (int)N2 - 1 && k > 0 &&
+                               k < (int)N3 - 1 && per4 && ctl;
+            if (inner) {
+                // every neighbour is a grid value: the operations of
+                // cell_value in the same order, with the upwind x and y
+                // neighbours loaded only and the ghosts' FP64 arithmetic out of
+                // the way (60x60x20x36: 50 -> 37 us per step; 128x128x64x96,
+                // bound by the FP64 unit: 1.47 -> 1.245 ms)
+                const T u1 = vin[nonneg(sc.w1) ? o + s1 : o - s1];
+                const T u2 = vin[nonneg(sc.w2) ? o + s2 : o - s2];
+                const T u3 = hj_max(vin[o + s3], vin[o - s3]);
+                const T u4 = hj_max(vin[l < (int)N4 - 1 ? o + 1 : o - l], vin[l > 0 ? o - 1 : o + (N4 - 1)]);
+                T r = sc.w0 * vc;
+                r = fma(mag(sc.w1), u1, r);
+                r = fma(mag(sc.w2), u2, r);
+                r = fma(k3dt, u3, r);
+                vn = fma(sc.w4, u4, r);
+            } else {
+                const Neigh<T> nx = axis_neighbours<T>(vin, o, cl.i, N1, s1, g.periodic & 1, vc);
+                const Neigh<T> ny = axis_neighbours<T>(vin, o, cl.j, N2, s2, (g.periodic >> 1) & 1, vc);
+                const Neigh<T> nv = axis_neighbours<T>(vin, o, k, N3, s3, (g.periodic >> 2) & 1, vc);
+                const Neigh<T> nt = axis_neighbours<T>(vin, o, l, N4, 1, (g.periodic >> 3) & 1, vc);
+                vn = cell_value(vc, nx, ny, nv, nt, sc, k3dt, g.mode3, g.mode4);
+            }
         } else {
-            const T u1 = nonneg(cf.c1) ? nx.p : nx.m;
-            const T u2 = nonneg(cf.c2) ? ny.p : ny.m;
-            const T K1 = fabs(cf.c1), K2 = fabs(cf.c2);
-            T r = K1 * (u1 - vc);
-            r = fmaf(K2, u2 - vc, r);
-            r = fmaf(k3, u3 - vc, r);
-            r = fmaf(((const float2 *)k4tab)[k].x, u4 - vc, r);  // theta coefficient of this speed
-            vn = fmaf(dt, r, vc);
+            const Neigh<T> nx = axis_neighbours<T>(vin, o, cl.i, N1, s1, g.periodic & 1, vc);
+            const Neigh<T> ny = axis_neighbours<T>(vin, o, cl.j, N2, s2, (g.periodic >> 1) & 1, vc);
+            const Neigh<T> nv = axis_neighbours<T>(vin, o, k, N3, s3, (g.periodic >> 2) & 1, vc);
+            const Neigh<T> nt = axis_neighbours<T>(vin, o, l, N4, 1, (g.periodic >> 3) & 1, vc);
+            const HjCoef<T> cf = coef[k * N4 + l];
+            vn = cell_value(vc, nx, ny, nv, nt, cf.c1, cf.c2, k3, ((const float2 *)k4tab)[k].x, dt, g.mode3, g.mode4);
         }
         vn = hj_min(v0[o], vn);  // BRT min with the target (Algorithm 2)
         vout[o] = vn;
-        if constexpr (TRACK) {  // convergence mode: largest change of V (Algorithm 2's epsilon)
-            if constexpr (sizeof(T) == 8) {
-                const unsigned long long b = hj_abits(mag(vn - vc));
-                dbits = dbits > b ? dbits : b;
-            } else {
-                dmf = fmaxf(dmf, fabsf(vn - vc));
-            }
-        }
-
-        // alpha_d^max: the largest |xdot_d| among the cells this thread updated
-        // (integer max of the FP64 bit patterns, in both precisions)
-        {
-            const unsigned long long b1 = hj_abits(cf.a1), b2 = hj_abits(cf.a2);
-            am1 = am1 > b1 ? am1 : b1;
-            am2 = am2 > b2 ? am2 : b2;
-        }
+        if constexpr (TRACK) track_change(mx, vn, vc);  // convergence mode: largest change of V
     }
-    if constexpr (sizeof(T) == 4) {
-        hj_step_epilogue(st, g, am1, am2, hj_abits((double)dmf), scratch);
-    } else {
-        hj_step_epilogue_scaled(st, g, am1, am2, dbits, scratch, scaled, nullptr, (const HjCoef<double> *)coef,
-                                (const double *)k4tab);
-    }
+    if constexpr (TRACK) hj_track_epilogue(lp, step_max_bits<T>(mx), scratch);
 }
 
 // ------------------------------------------------------------ resident form
@@ -427,14 +366,10 @@ __global__ void __launch_bounds__(256) hj_step_generic_kernel(const T *__restric
 // updates theta quads (4 consecutive cells of a row: one 16- or 32-byte load
 // per neighbour row instead of four) with the per-cell functions above, so
 // the results equal the per-step kernels' bit for bit.  Per CTA, in shared
-// memory: the loop state and the per-(v, theta) coefficients of the current
-// dt (rebuilt by the CTA itself when dt changes).  alpha^max does not depend
-// on V, so every CTA reduces it once from the coefficient table (the same
-// maximum as over the grid's cells); each step then needs one grid barrier
-// (plus a max-reduction of the change of V in convergence mode), after which
-// every CTA runs the finaliser on its copy of the state (identical inputs,
-// identical dt).  The state goes back to global memory at the end; a barrier
-// that times out records HJ_ERR_TIMEOUT and ends the launch.
+// memory: the per-(v, theta) coefficients of the current dt (rebuilt by the
+// CTA itself for the cut last step).  Each step needs one grid barrier (plus
+// a max-reduction of the change of V in convergence mode).  A barrier that
+// times out records HJ_ERR_TIMEOUT and ends the launch.
 
 constexpr int RES_THREADS = 256;
 constexpr int RES_MAX_PER_SM = 4;
@@ -651,15 +586,14 @@ constexpr int res_min_blocks()
 template <typename T, bool TRACK>
 __global__ void __launch_bounds__(RES_THREADS, res_min_blocks<T>()) hj_step_resident_kernel(
     const T *__restrict__ v0, T *buf, const void *__restrict__ coefp, const void *__restrict__ k4tab,
-    HjDevState *st, const HjGeom g, long long nint, const QuadDivisors dv, HjResidentSync *sync, long long ksteps,
-    unsigned long long limit_ns)
+    HjLoop *lp, HjFlags *flags, const HjGeom g, long long nint, const QuadDivisors dv, HjResidentSync *sync,
+    long long n0, long long ksteps, int cut, unsigned long long limit_ns)
 {
     constexpr bool Q = std::is_same<T, int32_t>::value;
     constexpr bool F32 = std::is_same<T, float>::value;
     extern __shared__ __align__(16) unsigned char res_smem[];
-    __shared__ HjDevState s;
-    __shared__ unsigned long long scratch[96];
-    __shared__ double s_alpha[2];
+    __shared__ unsigned long long scratch[32];
+    __shared__ double s_eps;
     __shared__ int s_ok;
 
     const int N1 = g.n1, N2 = g.n2, N3 = g.n3, N4 = g.n4, P4 = g.p4, tot = N3 * P4;
@@ -671,9 +605,6 @@ __global__ void __launch_bounds__(RES_THREADS, res_min_blocks<T>()) hj_step_resi
     double *w1t = (double *)res_smem, *w2t = w1t + tot, *w0t = w2t + tot, *w4t = w0t + tot;
     int32_t *qtab = (int32_t *)res_smem;
 
-    if (threadIdx.x == 0) s = *st;
-    // alpha^max over the coefficient table (= over the grid's cells)
-    unsigned long long a1 = 0ull, a2 = 0ull, dz = 0ull;
     if constexpr (F32) {
         const HjCoef<float> *coef = (const HjCoef<float> *)coefp;
         for (int e = threadIdx.x; e < tot; e += blockDim.x) {
@@ -683,41 +614,14 @@ __global__ void __launch_bounds__(RES_THREADS, res_min_blocks<T>()) hj_step_resi
                 const HjCoef<float> c = coef[k * N4 + l];
                 c1 = c.c1;
                 c2 = c.c2;
-                const unsigned long long b1 = hj_abits(c.a1), b2 = hj_abits(c.a2);
-                a1 = a1 > b1 ? a1 : b1;
-                a2 = a2 > b2 ? a2 : b2;
             }
             c1t[e] = c1;
             c2t[e] = c2;
         }
         for (int k = threadIdx.x; k < N3; k += blockDim.x) k4s[k] = ((const float2 *)k4tab)[k].x;
-    } else {
-        const HjCoef<double> *coef = (const HjCoef<double> *)coefp;
-        for (int e = threadIdx.x; e < N3 * N4; e += blockDim.x) {
-            const unsigned long long b1 = hj_abits(coef[e].a1), b2 = hj_abits(coef[e].a2);
-            a1 = a1 > b1 ? a1 : b1;
-            a2 = a2 > b2 ? a2 : b2;
-        }
+        __syncthreads();
     }
-    hj_block_max3(a1, a2, dz, scratch);
-    if (threadIdx.x == 0) {
-        s_alpha[0] = __longlong_as_double((long long)a1);
-        s_alpha[1] = __longlong_as_double((long long)a2);
-    }
-    __syncthreads();
-    double table_dt = 0.0;  // dt the FP64 / Q5.27 table holds (0: not built)
-    if constexpr (!F32) {
-        if (!s.done) {
-            if constexpr (Q)
-                hj_rescale_qweights(qtab, (const HjCoef<double> *)coefp, N3, N4, P4, g.k3, (const double *)k4tab,
-                                    s.dt);
-            else
-                resident_table64(w1t, w2t, w0t, w4t, (const HjCoef<double> *)coefp, (const double *)k4tab, N3, N4,
-                                 P4, s.dt);
-            table_dt = s.dt;
-            __syncthreads();
-        }
-    }
+    double table_dt = -1.0;  // dt the FP64 / Q5.27 table holds (negative: not built)
 
     const long long s2 = (long long)N3 * P4, s1 = (long long)N2 * s2;
     const unsigned int Q4 = (unsigned int)(P4 / 4);
@@ -726,13 +630,25 @@ __global__ void __launch_bounds__(RES_THREADS, res_min_blocks<T>()) hj_step_resi
     const unsigned long long qstride = (unsigned long long)gridDim.x * blockDim.x;
     const bool per4 = (per >> 3) & 1;
     unsigned int barriers = 0;
-    bool aborted = false;
-    for (long long it = 0; it < ksteps && !s.done; ++it) {
+    for (long long it = 0; it < ksteps; ++it) {
         const T *vin;
         T *vout;
-        hj_io_buffers<T>(v0, buf, nint, s.n, vin, vout);
-        const T dt = (T)s.dt;
-        const double k3dt = g.k3 * s.dt;
+        hj_io_buffers<T>(v0, buf, nint, n0 + it, vin, vout);
+        const double dtd = lp->dt[cut && it == ksteps - 1 ? 1 : 0];
+        const T dt = (T)dtd;
+        const double k3dt = g.k3 * dtd;
+        if constexpr (!F32) {
+            if (dtd != table_dt) {  // the first step and the cut last one (the barrier freed the old table)
+                if constexpr (Q)
+                    hj_rescale_qweights(qtab, (const HjCoef<double> *)coefp, N3, N4, P4, g.k3, (const double *)k4tab,
+                                        dtd, threadIdx.x, blockDim.x);
+                else
+                    resident_table64(w1t, w2t, w0t, w4t, (const HjCoef<double> *)coefp, (const double *)k4tab, N3, N4,
+                                     P4, dtd);
+                table_dt = dtd;
+                __syncthreads();
+            }
+        }
         StepMax m;
         for (unsigned long long q = q0; q < nquad; q += qstride) {
             const uint32_t q32 = (uint32_t)q, row = fast_div(q32, dv.q4);
@@ -844,60 +760,35 @@ __global__ void __launch_bounds__(RES_THREADS, res_min_blocks<T>()) hj_step_resi
         }
         unsigned long long *slot = &sync->slot[(int)(it % 3)];
         if constexpr (TRACK) {  // the step's largest change of V, grid-wide
-            unsigned long long u1 = 0ull, u2 = 0ull, d;
-            step_max_bits<T>(m, u1, u2, d);
-            hj_block_max3(u1, u2, d, scratch);
+            const unsigned long long d = hj_block_max(step_max_bits<T>(m), scratch);
             if (threadIdx.x == 0 && d) atomicMax(slot, d);
         }
         ++barriers;
         if (!hj_grid_sync(&sync->count, gridDim.x * barriers, limit_ns, &s_ok)) {
-            aborted = true;
-            break;
+            if (threadIdx.x == 0) *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
+            return;
         }
-        if (threadIdx.x == 0) {
-            double eps = 0.0;
-            if constexpr (TRACK) {
-                eps = __longlong_as_double((long long)__ldcg(slot));
-                // the slot of step it - 1 is read by every CTA by now: clear it for step it + 2
-                if (blockIdx.x == 0) sync->slot[(int)((it + 2) % 3)] = 0ull;
+        if constexpr (TRACK) {
+            if (threadIdx.x == 0) {
+                s_eps = __longlong_as_double((long long)__ldcg(slot));
+                if (blockIdx.x == 0) {
+                    // the slot of step it - 1 was read by every CTA before this barrier: clear it for step it + 2
+                    sync->slot[(int)((it + 2) % 3)] = 0ull;
+                    lp->delta_last = s_eps;
+                    lp->taken = it + 1;
+                }
             }
-            hj_finalise_values(&s, g, s_alpha[0], s_alpha[1], eps);
-        }
-        __syncthreads();
-        if constexpr (!F32) {
-            if (!s.done && s.dt != table_dt) {  // after the first step and before the cut last one
-                if constexpr (Q)
-                    hj_rescale_qweights(qtab, (const HjCoef<double> *)coefp, N3, N4, P4, g.k3,
-                                        (const double *)k4tab, s.dt);
-                else
-                    resident_table64(w1t, w2t, w0t, w4t, (const HjCoef<double> *)coefp, (const double *)k4tab, N3,
-                                     N4, P4, s.dt);
-                table_dt = s.dt;
-                __syncthreads();
+            __syncthreads();
+            if (s_eps < lp->threshold) {  // Algorithm 2's convergence test
+                if (threadIdx.x == 0 && blockIdx.x == 0) lp->done = 1;
+                return;
             }
         }
-    }
-    if (threadIdx.x != 0) return;
-    if (aborted) {
-        atomicCAS(&st->status, (int)HJ_OK, (int)HJ_ERR_TIMEOUT);
-        return;
-    }
-    if (blockIdx.x == 0) {  // every CTA holds the same state; the global tables were not touched
-        st->t = s.t;
-        st->dt = s.dt;
-        st->dt_prev = s.dt_prev;
-        st->n = s.n;
-        st->last = s.last;
-        st->done = s.done;
-        for (int d = 0; d < 4; ++d) st->alpha_prev[d] = s.alpha_prev[d];
-        st->converged = s.converged;
-        st->delta_last = s.delta_last;
-        if (s.status != HJ_OK) atomicCAS(&st->status, (int)HJ_OK, s.status);
     }
 }
 
 template <typename T, bool TRACK>
-cudaError_t launch_resident(hj_grid *g, long long k)
+cudaError_t launch_resident(hj_grid *g, long long n, long long k, bool cut)
 {
     const void *fn = (const void *)hj_step_resident_kernel<T, TRACK>;
     const size_t smem = resident_table_bytes(g);
@@ -921,13 +812,14 @@ cudaError_t launch_resident(hj_grid *g, long long k)
     T *buf = (T *)g->buf;
     const void *coef = g->coef;
     const void *k4 = g->k4tab;
-    HjDevState *st = g->dstate;
+    HjLoop *lp = g->loop;
+    HjFlags *flags = g->dflags;
     HjGeom geom = g->geom;
-    long long nint = g->nint;
+    long long nint = g->nint, n0 = n, ksteps = k;
     HjResidentSync *sync = g->rsync;
-    long long ksteps = k;
+    int cut_last = cut ? 1 : 0;
     unsigned long long limit = RES_WAIT_NS;
-    void *args[] = {&v0, &buf, &coef, &k4, &st, &geom, &nint, &dv, &sync, &ksteps, &limit};
+    void *args[] = {&v0, &buf, &coef, &k4, &lp, &flags, &geom, &nint, &dv, &sync, &n0, &ksteps, &cut_last, &limit};
     return cudaLaunchCooperativeKernel(fn, blocks, RES_THREADS, args, smem, g->stream);
 }
 
@@ -940,7 +832,7 @@ bool hj_resident_supported(const hj_grid *g)
     return coop != 0 && g->nint < (1LL << 32) && resident_table_bytes(g) <= RES_MAX_TABLE;
 }
 
-cudaError_t hj_launch_step_resident(hj_grid *g, long long k)
+cudaError_t hj_launch_step_resident(hj_grid *g, long long n, long long k, bool cut)
 {
     if (!g->rsync) {
         cudaError_t e = cudaMalloc(&g->rsync, sizeof(HjResidentSync));
@@ -952,9 +844,9 @@ cudaError_t hj_launch_step_resident(hj_grid *g, long long k)
     }
     cudaError_t e = cudaMemsetAsync(g->rsync, 0, sizeof(HjResidentSync), g->stream);
     if (e != cudaSuccess) return e;
-    if (g->prec == HJ_Q527) return g->track ? launch_resident<int32_t, true>(g, k) : launch_resident<int32_t, false>(g, k);
-    if (g->prec == HJ_FP64) return g->track ? launch_resident<double, true>(g, k) : launch_resident<double, false>(g, k);
-    return g->track ? launch_resident<float, true>(g, k) : launch_resident<float, false>(g, k);
+    if (g->prec == HJ_Q527) return g->track ? launch_resident<int32_t, true>(g, n, k, cut) : launch_resident<int32_t, false>(g, n, k, cut);
+    if (g->prec == HJ_FP64) return g->track ? launch_resident<double, true>(g, n, k, cut) : launch_resident<double, false>(g, n, k, cut);
+    return g->track ? launch_resident<float, true>(g, n, k, cut) : launch_resident<float, false>(g, n, k, cut);
 }
 
 // Launch of a step kernel as a programmatic dependent of the previous launch
@@ -975,7 +867,7 @@ static cudaError_t launch_dependent(void (*fn)(KArgs...), int blocks, int thread
     return cudaLaunchKernelEx(&cfg, fn, (KArgs)args...);
 }
 
-cudaError_t hj_launch_step_generic(hj_grid *g)
+cudaError_t hj_launch_step_generic(hj_grid *g, long long n, int sel)
 {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
@@ -990,14 +882,17 @@ cudaError_t hj_launch_step_generic(hj_grid *g)
     dv.n2 = make_fastdiv((uint32_t)g->n[1]);
     const bool fast = g->ncell < (1LL << 32);
     cudaError_t le = cudaSuccess;
-#define HJ_LAUNCH_Q(F, K)                                                                                      \
-    le = launch_dependent(hj_step_q527_kernel<F, K>, blocks, threads, g->stream, (const int32_t *)g->v0,      \
-                          (int32_t *)g->buf, (const HjCoef<double> *)g->coef, g->qw, (const double *)g->k4tab, \
-                          g->dstate, g->geom, g->nint, dv)
-#define HJ_LAUNCH(T, F, K)                                                                                     \
-    le = launch_dependent(hj_step_generic_kernel<T, F, K>, blocks, threads, g->stream, (const T *)g->v0,      \
-                          (T *)g->buf, (const HjCoef<T> *)g->coef, g->scaled, (const void *)g->k4tab, g->dstate, \
-                          g->geom, g->nint, dv)
+    const void *vin = hj_value_ptr(g, n);
+    void *vout = hj_value_ptr(g, n + 1);
+    const HjScaledCoef *scaled = g->scaled ? g->scaled + (size_t)sel * g->n[2] * g->n[3] : nullptr;
+    const int32_t *qw = g->qw ? g->qw + sel * hj_qw_count(g->n[2], g->p4) : nullptr;
+#define HJ_LAUNCH_Q(F, K)                                                                                        \
+    le = launch_dependent(hj_step_q527_kernel<F, K>, blocks, threads, g->stream, (const int32_t *)g->v0,        \
+                          (const int32_t *)vin, (int32_t *)vout, qw, g->loop, g->geom, dv)
+#define HJ_LAUNCH(T, F, K)                                                                                       \
+    le = launch_dependent(hj_step_generic_kernel<T, F, K>, blocks, threads, g->stream, (const T *)g->v0,        \
+                          (const T *)vin, (T *)vout, (const HjCoef<T> *)g->coef, scaled, (const void *)g->k4tab, \
+                          g->loop, sel, g->geom, dv)
 #define HJ_LAUNCH2(T, F)          \
     do {                          \
         if (g->track)             \

@@ -102,7 +102,7 @@ int best_chunk(const hj_grid *g, int ncol, int slots)
 
 size_t tiled_smem_bytes(const TiledParams &P)
 {
-    return (size_t)P.stages * P.stage_bytes + 2 * MAX_STAGES * sizeof(uint64_t) + 96 * sizeof(unsigned long long) +
+    return (size_t)P.stages * P.stage_bytes + 2 * MAX_STAGES * sizeof(uint64_t) + 32 * sizeof(unsigned long long) +
            32;
 }
 
@@ -281,7 +281,7 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
     return true;
 }
 
-cudaError_t hj_launch_step_tiled(hj_grid *g)
+cudaError_t hj_launch_step_tiled(hj_grid *g, long long n, int sel)
 {
     const TiledParams P = make_params(g, g->tile_ty, g->tile_tv, g->tile_stages, g->tile_xc);
     KernelFn fn =
@@ -299,7 +299,9 @@ cudaError_t hj_launch_step_tiled(hj_grid *g)
     cfg.stream = g->stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fn, g->tmap[0], g->tmap[1], g->tmap[2], g->tmap[3], (float *)g->buf,
-                              (const void *)g->coef, (const float *)g->tab_tiled, g->qw, (const float *)g->v0xy,
-                              (const void *)g->k4tab, (const double2 *)g->amax_q, g->dstate, g->geom, P, g->nint);
+    const CUtensorMap &in = n == 0 ? g->tmap[0] : g->tmap[1 + (int)((n - 1) & 1)];
+    const int32_t *qw = g->qw ? g->qw + sel * hj_qw_count(g->n[2], g->p4) : nullptr;
+    return cudaLaunchKernelEx(&cfg, fn, in, g->tmap[3], (float *)hj_value_ptr(g, n + 1), (const float *)g->tab_tiled,
+                              qw, (const float *)g->v0xy, (const void *)g->k4tab, g->loop, sel, g->dflags, g->geom,
+                              P);
 }

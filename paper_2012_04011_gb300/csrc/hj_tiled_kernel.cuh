@@ -22,17 +22,15 @@
 //     by shared memory and L2.
 //   * All CTAs of a step sweep x concurrently, so y/v halo rows of
 //     neighbouring columns are in L2 when they are needed.
-//   * alpha^max partials (|xdot_1|, |xdot_2| over the (v, theta) states of the
-//     cells each thread updates: one FP64 pair per (v, theta quad) of each of
-//     its items, from a small table) are reduced by each consumer thread at
-//     the start, while the first planes are in flight, then by warp shuffles
-//     and shared-memory maxima; the last CTA computes the next CFL step
-//     (fused; no extra pass over the grid, no registers held in the sweep).
+//   * No reductions, atomics or shared state between the CTAs of a step:
+//     alpha^max does not depend on V (Sec. II-B of the paper), so the host
+//     runs the time loop and a step only reads its dt (HjLoop).  A per-step
+//     alpha^max reduction and last-CTA finaliser cost 2.7 of 66.9 ms over the
+//     352 steps of a 128x128x64x96 solve.
 // The Q5.27 variant (FIXED) moves the same 4-byte values through the same
 // ring and evaluates the fixed-point update of hj_q527_update per lane:
 // exact integer upwind differences (ghosts by flag, as minus the difference
-// on the other side), per-(v, theta) weights from the fixed-point table, and
-// the FP64 coefficient table for alpha^max.
+// on the other side) and per-(v, theta) weights from the fixed-point table.
 // Broadcast V0 (BCAST): when V0 depends on (x, y) only (Eq. init_V), the
 // grid keeps its N1 x N2 field and the kernel reads V0 from it (one scalar
 // per row and plane, an L1/L2 hit) instead of a V0 box per plane: 8
@@ -47,7 +45,7 @@
 // times the tile; that L2 traffic, not the arithmetic, sets the pace of this
 // variant.  Each cell's arithmetic is the one-row form's, in the same order.
 // Every mbarrier wait is bounded by %globaltimer; on timeout the kernel
-// records HJ_ERR_TIMEOUT in the device state, stops issuing work, waits
+// records HJ_ERR_TIMEOUT in the grid's flags, stops issuing work, waits
 // (bounded) for its own copies in flight and returns.
 #pragma once
 
@@ -55,7 +53,6 @@
 #include <stdio.h>
 #include <string.h>
 
-#include "hj_scaled.cuh"
 #include "hj_tma.cuh"
 
 // The kernel template lives in this header; hj_tiled_f32.cu,
@@ -127,15 +124,13 @@ __device__ __forceinline__ int32_t f4geti(const float4 &v, int e) { return __flo
 // RPT: v rows per consumer thread (2 or 4 only with BCAST, USIGN, FP32, unpadded).
 template <bool FIXED, bool PADDED, bool USIGN, bool BCAST, bool TRACK, int MAXC, int RPT = 1>
 __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
-    const __grid_constant__ CUtensorMap map_v0, const __grid_constant__ CUtensorMap map_a,
-    const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_v0_tile,
-    float *__restrict__ buf, const void *__restrict__ coefv, const float *__restrict__ tab,
-    int32_t *__restrict__ qw, const float *__restrict__ v0xy, const void *__restrict__ k4tab,
-    const double2 *__restrict__ amaxq, HjDevState *st, const HjGeom g, const TiledParams P, long long nint)
+    const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_v0_tile,
+    float *__restrict__ vout, const float *__restrict__ tab, const int32_t *__restrict__ qw,
+    const float *__restrict__ v0xy, const void *__restrict__ k4tab, HjLoop *lp, int sel, HjFlags *flags,
+    const HjGeom g, const TiledParams P)
 {
     static_assert(RPT == 1 || ((RPT == 2 || RPT == 4) && BCAST && USIGN && !FIXED && !PADDED),
                   "several rows per thread: broadcast V0, single-sided FP32");
-    const HjCoef<double> *coefd = (const HjCoef<double> *)coefv;  // Q5.27 grids: the table the weights come from
     extern __shared__ __align__(1024) unsigned char smem_raw[];
 
     // ---- shared memory carve-up
@@ -143,9 +138,8 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
     uint64_t *full = (uint64_t *)(smem_raw + (size_t)P.stages * P.stage_bytes);
     uint64_t *empty = full + MAX_STAGES;
     unsigned long long *scratch = (unsigned long long *)(empty + MAX_STAGES);
-    volatile int *abort_flag = (volatile int *)(scratch + 96);
-    unsigned long long *deadline_p = (unsigned long long *)(scratch + 97);
-    unsigned long long *alpha_s = scratch + 98;  // the CTA's alpha^max partials (FP64 bit patterns)
+    volatile int *abort_flag = (volatile int *)(scratch + 32);
+    unsigned long long *deadline_p = (unsigned long long *)(scratch + 33);
 
     const int tid = threadIdx.x;
     const int nconsumer_warps = P.nconsumer >> 5;
@@ -156,24 +150,19 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
         }
         *abort_flag = 0;
         *deadline_p = global_ns() + HJ_WAIT_NS;
-        alpha_s[0] = 0ull;
-        alpha_s[1] = 0ull;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
     // Launched as a programmatic dependent of the previous step (the host sets
     // the launch attribute): everything above overlaps that step's end; from
-    // here on the previous grid has completed and its V_n and finalised state
-    // are visible.  Then the next step may be scheduled as SMs free up (its
-    // CTAs wait here in turn).  Without such a prerequisite both are no-ops.
+    // here on the previous grid has completed and its V_n is visible.  Then
+    // the next step may be scheduled as SMs free up (its CTAs wait here in
+    // turn).  Without such a prerequisite both are no-ops.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (st->done) return;  // uniform across the grid
+    if (TRACK && lp->done) return;  // uniform across the grid
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long n = st->n;
-    const float dt = (float)st->dt;
-    float *vout = buf + (n & 1) * nint;
-    const CUtensorMap *map_in = (n == 0) ? &map_v0 : (((n - 1) & 1) ? &map_b : &map_a);
+    const float dt = (float)lp->dt[sel];
 
     // convergence mode (Algorithm 2's epsilon): this thread's largest |V_{n+1} - V_n|
     float dmf = 0.f;
@@ -208,7 +197,7 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
                     const bool interior = !BCAST && p >= it.x0 && p < it.x1;
                     float *dst = stages + (size_t)slot * (P.stage_bytes / 4);
                     mbar_arrive_expect_tx(&full[slot], tx_halo + (interior ? tx_v0 : 0u));
-                    tma_load_4d(dst, map_in, &full[slot], 0, it.v0 - 1, it.y0 - 1, p);
+                    tma_load_4d(dst, &map_in, &full[slot], 0, it.v0 - 1, it.y0 - 1, p);
                     if (interior) tma_load_4d(dst + P.halo_floats, &map_v0_tile, &full[slot], 0, it.v0, it.y0, p);
                     used_mask |= 1u << slot;
                     last_phase = (last_phase & ~(1u << slot)) | (phase << slot);
@@ -220,14 +209,14 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
                 }
             }
             if (!ok) {
-                st->status = HJ_ERR_TIMEOUT;
+                *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
                 *abort_flag = 1;
             }
             // drain: every copy this CTA issued must land before the CTA exits
             const unsigned long long drain_deadline = global_ns() + HJ_WAIT_NS;
             for (int s = 0; s < P.stages; ++s)
                 if (((used_mask >> s) & 1u) && !mbar_wait(&full[s], (last_phase >> s) & 1u, drain_deadline))
-                    st->status = HJ_ERR_TIMEOUT;
+                    *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
         }
     } else {
         // ------------------------------------------------------------ consumers
@@ -242,32 +231,6 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
         const int tvr = RPT == 1 ? P.tv : P.tv / RPT;  // threads along v (the host makes tv a multiple of RPT)
         const int jy = r / tvr, kv = (r - jy * tvr) * RPT;
         const bool inrow = r < P.ty * tvr;
-        {
-            // alpha^max partials: the FP64 |xdot_1|, |xdot_2| maxima over this
-            // thread's theta quad in the row it owns in each of its items (the
-            // car's velocity depends on v and theta only), reduced while the
-            // producer's first copies are in flight
-            unsigned long long ab1 = 0ull, ab2 = 0ull;
-#pragma unroll 4
-            for (int item = blockIdx.x; item < P.nitems; item += gridDim.x) {
-                const int col = item % P.ncol;
-                const int y = (col / P.ncol_v) * P.ty + jy, v = (col % P.ncol_v) * P.tv + kv;
-#pragma unroll
-                for (int rr = 0; rr < RPT; ++rr)
-                    if (inrow && y < g.n2 && v + rr < g.n3) {
-                        const double2 am = amaxq[(v + rr) * P.q4 + q];
-                        const unsigned long long b1 = hj_abits(am.x), b2 = hj_abits(am.y);
-                        ab1 = ab1 > b1 ? ab1 : b1;
-                        ab2 = ab2 > b2 ? ab2 : b2;
-                    }
-            }
-            ab1 = hj_warp_max_u64(ab1);
-            ab2 = hj_warp_max_u64(ab2);
-            if (lane == 0) {
-                atomicMax(&alpha_s[0], ab1);
-                atomicMax(&alpha_s[1], ab2);
-            }
-        }
         const int rsm = inrow ? ((jy + 1) * srow + (kv + 1)) * P4 + 4 * q : (srow + 1) * P4;
         const int r0sm = P.halo_floats + (inrow ? (jy * P.tv + kv) * P4 + 4 * q : 0);  // V0 in the stage
         // V_{n+1} is addressed in float4 units (P4 is a multiple of 4): 32-bit
@@ -680,23 +643,18 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
 #undef HJ_WAIT_NEXT
 #undef HJ_RELEASE_OLDEST
         if (!ok) {
-            st->status = HJ_ERR_TIMEOUT;
+            *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
             *abort_flag = 1;
         }
     }
-    // the CTA's alpha^max partials enter the block reduction through thread 0
-    __syncthreads();
-    const unsigned long long ab1 = tid == 0 ? alpha_s[0] : 0ull, ab2 = tid == 0 ? alpha_s[1] : 0ull;
-    if constexpr (FIXED)
-        hj_step_epilogue_scaled(st, g, ab1, ab2, hj_abits((double)dmq * (1.0 / HJ_Q527_SCALE)), scratch, nullptr, qw,
-                                coefd, (const double *)k4tab);
-    else
-        hj_step_epilogue(st, g, ab1, ab2, hj_abits((double)dmf), scratch);
+    if constexpr (TRACK) {
+        __syncthreads();
+        hj_track_epilogue(lp, FIXED ? hj_abits((double)dmq * (1.0 / HJ_Q527_SCALE)) : hj_abits((double)dmf), scratch);
+    }
 }
 
-typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, float *,
-                         const void *, const float *, int32_t *, const float *, const void *, const double2 *,
-                         HjDevState *, const HjGeom, const TiledParams, long long);
+typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, float *, const float *, const int32_t *, const float *,
+                         const void *, HjLoop *, int, HjFlags *, const HjGeom, const TiledParams);
 
 // Kernel of a variant, smallest launch bound class that holds nconsumer
 // consumer threads (defined in the instantiating translation units); rpt is
