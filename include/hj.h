@@ -118,8 +118,10 @@ typedef enum {
     HJ_KERNEL_RESIDENT = 3 /* the per-cell update of HJ_KERNEL_GENERIC (identical results, any
                             * precision and grid of fewer than 2^32 values whose coefficient
                             * tables fit in shared memory), the whole time loop in one
-                            * cooperative launch with a grid barrier between steps; a barrier
-                            * wait that runs out (2 s) ends the call with HJ_ERR_TIMEOUT */
+                            * cooperative launch with a grid barrier between steps, or, for FP32
+                            * and Q5.27 car grids that fit, with the values held in the SMs'
+                            * shared memory and waits between neighbouring blocks only; a wait
+                            * that runs out (2 s) ends the call with HJ_ERR_TIMEOUT */
 } hj_kernel;
 
 typedef struct {

@@ -320,7 +320,8 @@ void reset_state(hj_grid *g)
 // Whether HJ_KERNEL_AUTO takes the resident kernel: FP32 grids of up to 4 M
 // cells and Q5.27 grids of up to 8 M cells (measured crossovers against the
 // tiled kernel), where a step takes a few microseconds and the per-step
-// launch and last-CTA finaliser of the other kernels cost about as much.
+// launches of the other kernels cost about as much.  (Within them a grid whose
+// blocks fit on chip runs the on-chip form, hj_onchip.cuh.)
 // Larger grids stream faster through the tiled kernel; FP64 steps are bound
 // by the FP64 unit, where the resident form gains nothing.
 bool resident_auto(const hj_grid *g)
@@ -698,6 +699,7 @@ hj_status hj_set_dynamics(hj_grid *g, hj_dynamics kind, const double *params, in
     char why[160];
     g->tiled_ok = hj_tiled_setup(g, why, sizeof(why));
     if (g->kernel_req == HJ_KERNEL_TILED && !g->tiled_ok) g->kernel_req = HJ_KERNEL_AUTO;
+    hj_onchip_setup(g);
     // a previously set V0 stays; the next solve continues with the new dynamics
     return HJ_OK;
 }

@@ -66,14 +66,19 @@ struct HjScaledCoef {
     double w1, w2, w0, w4;  // w4 = dt |xdot_4| / dx_4 (depends on v for the steering car)
 };
 
-// Device-side bookkeeping of the resident step kernel: the grid barrier's
-// arrival counter and three rotating slots of the per-step largest change
-// of V (convergence mode; FP64 bit patterns).  Zeroed before every resident
-// launch.
+// Device-side bookkeeping of the resident and on-chip step kernels: the grid
+// barrier's arrival counter, three rotating slots of the per-step largest
+// change of V (convergence mode; FP64 bit patterns), and the steps each CTA of
+// the on-chip kernel has published.  Zeroed before every such launch.
+// (one 128-byte line per CTA: with the counters packed, the CTAs' polls queue up
+// on a few lines and a step's wait takes 4.5 us instead of 1.2).
+constexpr int HJ_SYNC_CTAS = 512;
+constexpr int HJ_SYNC_STRIDE = 32;
 struct HjResidentSync {
     unsigned int count;
     unsigned int unused;
     unsigned long long slot[3];
+    unsigned int prog[HJ_SYNC_CTAS * HJ_SYNC_STRIDE] __attribute__((aligned(128)));
 };
 
 // Grid geometry handed to kernels by value.
@@ -144,7 +149,9 @@ struct hj_grid {
     int32_t tile_req[4];   // requested (ty, tv, xc, stages); 0 = choose automatically
     int32_t tile_ty, tile_tv, tile_xc, tile_stages;
     int32_t tiled_ctas, tiled_per_sm;
-    bool tiled_usign;      // every theta quad has one sign of cos and of sin
+    bool tiled_usign;      // FP32: every theta quad has one sign of cos and of sin, and every speed is >= 0
+    int oc_bx, oc_by;      // on-chip kernel: columns of a block along x and y (0: not used)
+    bool sign_uniform;     // every theta quad has one sign of cos and of sin (lanes flushed to 0 count as either)
 
     cudaEvent_t ev[4];
     // CUDA graphs of k back-to-back step launches (small grids, where the
@@ -170,6 +177,11 @@ cudaError_t hj_launch_step_tiled(hj_grid *g, long long n, int sel);
 // kernel, the last of them with dt[1] if cut (convergence mode: it stops early
 // when the test ends the loop); allocates g->rsync on first use.
 cudaError_t hj_launch_step_resident(hj_grid *g, long long n, long long k, bool cut);
+// The on-chip form of the resident kernel: choose the blocks for this grid
+// (oc_bx = 0: it does not take it), and its launch (as hj_launch_step_resident;
+// not in convergence mode).
+void hj_onchip_setup(hj_grid *g);
+cudaError_t hj_launch_onchip(hj_grid *g, long long n, long long k, bool cut);
 // Whether the device can run the resident kernel (cooperative launch).
 bool hj_resident_supported(const hj_grid *g);
 // Set up the tiled kernel for g (tensor maps, tile shape); false if unsupported.

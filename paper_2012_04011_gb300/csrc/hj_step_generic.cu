@@ -844,6 +844,7 @@ cudaError_t hj_launch_step_resident(hj_grid *g, long long n, long long k, bool c
     }
     cudaError_t e = cudaMemsetAsync(g->rsync, 0, sizeof(HjResidentSync), g->stream);
     if (e != cudaSuccess) return e;
+    if (!g->track && g->oc_bx > 0) return hj_launch_onchip(g, n, k, cut);
     if (g->prec == HJ_Q527) return g->track ? launch_resident<int32_t, true>(g, n, k, cut) : launch_resident<int32_t, false>(g, n, k, cut);
     if (g->prec == HJ_FP64) return g->track ? launch_resident<double, true>(g, n, k, cut) : launch_resident<double, false>(g, n, k, cut);
     return g->track ? launch_resident<float, true>(g, n, k, cut) : launch_resident<float, false>(g, n, k, cut);

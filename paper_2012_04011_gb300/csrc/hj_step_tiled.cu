@@ -180,7 +180,8 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
     if (!sgn) return fail("host allocation failed");
     // the single-sided (USIGN) form also needs every speed >= 0 (a negative
     // speed flips the upwind side); otherwise the general form runs
-    const bool usign = !fixed && g->lo[2] >= 0.0 && sign_uniform(g, sgn);
+    g->sign_uniform = sign_uniform(g, sgn);
+    const bool usign = !fixed && g->lo[2] >= 0.0 && g->sign_uniform;
     cudaError_t e = cudaMemcpy(g->tab_tiled + g->n[2] + 2 * g->p4, sgn, sizeof(float) * g->p4, cudaMemcpyHostToDevice);
     free(sgn);
     if (e != cudaSuccess) return fail("sign table upload failed");
