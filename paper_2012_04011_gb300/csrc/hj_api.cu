@@ -130,7 +130,7 @@ struct PrologueArgs {
 };
 
 __global__ void prologue_kernel(HjLoop *lp, const PrologueArgs a, const HjGeom g,
-                                const HjCoef<double> *__restrict__ coef, HjScaledCoef *scaled, int32_t *qw,
+                                const HjCoef<double> *__restrict__ coef, double *scaled, int32_t *qw,
                                 const double *__restrict__ k4)
 {
     const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
@@ -146,7 +146,8 @@ __global__ void prologue_kernel(HjLoop *lp, const PrologueArgs a, const HjGeom g
     }
     for (int i = 0; i < 2; ++i) {
         if (!a.build[i]) continue;
-        if (scaled) hj_rescale_table(scaled + (size_t)i * g.n3 * g.n4, coef, k4, g.n3, g.n4, a.dt[i], first, stride);
+        if (scaled) hj_rescale_table(scaled + i * hj_scaled_count(g.n3, g.p4), coef, k4, g.n3, g.n4, g.p4, a.dt[i], first,
+                             stride);
         else if (qw)
             hj_rescale_qweights(qw + i * hj_qw_count(g.n3, g.p4), coef, g.n3, g.n4, g.p4, g.k3, k4, a.dt[i], first,
                                 stride);
@@ -598,7 +599,7 @@ hj_status hj_create_grid(const int32_t n[4], const double lo[4], const double hi
     // FP64 coefficients for FP64 and Q5.27 grids (alpha^max and dt are FP64)
     const size_t coef_bytes = ncoef * (prec == HJ_FP32 ? sizeof(HjCoef<float>) : sizeof(HjCoef<double>));
     const size_t qw_bytes = prec == HJ_Q527 ? 2 * sizeof(int32_t) * hj_qw_count(n[2], g->p4) : 0;
-    const size_t scaled_bytes = prec == HJ_FP64 ? 2 * ncoef * sizeof(HjScaledCoef) : 0;
+    const size_t scaled_bytes = prec == HJ_FP64 ? 2 * sizeof(double) * hj_scaled_count(n[2], g->p4) : 0;
     const size_t k4_bytes = (size_t)n[2] * (prec == HJ_FP32 ? 2 * sizeof(float) : sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&g->coef, coef_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&g->tab_tiled, sizeof(float) * ((size_t)n[2] + 3 * (size_t)g->p4));

@@ -119,7 +119,7 @@ struct hj_grid {
     void *v0;              // V0 (internal layout)
     void *buf;             // two ping-pong buffers, back to back (2*nint values)
     void *coef;            // HjCoef<T>[n3*n4]
-    HjScaledCoef *scaled;  // FP64 grids: dt-scaled coefficients [n3*n4], one table per entry of HjLoop::dt
+    double *scaled;        // FP64 grids: dt-scaled coefficients (hj_rescale_table), one table per entry of HjLoop::dt
     int32_t *qw;           // Q5.27 grids: fixed-point axis weights (hj_rescale_qweights), likewise two tables
     void *k4tab;           // theta coefficient per speed: |xdot_4|/dx_4 (double[n3]; FP32 grids: float2[n3] of
                            // (k4, -(k3 + k4)))
@@ -231,12 +231,27 @@ __device__ __forceinline__ HjScaledCoef hj_scaled_entry(const HjCoef<double> &c,
     return o;
 }
 
-// The table for dt, n3 * n4 entries, by `stride` threads of which the caller
-// is number `first` (k4: the theta coefficient of each speed).
-__device__ __forceinline__ void hj_rescale_table(HjScaledCoef *sc, const HjCoef<double> *coef, const double *k4,
-                                                 int n3, int n4, double dt, int first, int stride)
+// The FP64 table for dt: w1, w2, w0 per (v, theta) as three arrays of n3 rows
+// of p4 entries (a pair of headings is one 16-byte load of each; pad entries
+// 0), then w4 per speed.  Filled by `stride` threads of which the caller is
+// number `first` (k4: the theta coefficient of each speed).
+__host__ __device__ __forceinline__ size_t hj_scaled_count(int n3, int p4)
 {
-    for (int i = first; i < n3 * n4; i += stride) sc[i] = hj_scaled_entry(coef[i], k4[i / n4], dt);
+    return (3 * (size_t)n3 * p4 + n3 + 1) / 2 * 2;
+}
+__device__ __forceinline__ void hj_rescale_table(double *sc, const HjCoef<double> *coef, const double *k4, int n3,
+                                                 int n4, int p4, double dt, int first, int stride)
+{
+    const int tot = n3 * p4;
+    for (int i = first; i < tot; i += stride) {
+        const int k = i / p4, l = i - k * p4;
+        HjScaledCoef o = {0.0, 0.0, 0.0, 0.0};
+        if (l < n4) o = hj_scaled_entry(coef[k * n4 + l], k4[k], dt);
+        sc[i] = o.w1;
+        sc[tot + i] = o.w2;
+        sc[2 * tot + i] = o.w0;
+    }
+    for (int k = first; k < n3; k += stride) sc[3 * tot + k] = dt * k4[k];
 }
 
 // ---- Q5.27 fixed point (Sec. III-C, Sec. IV-B): int32 codes q, value q 2^-27

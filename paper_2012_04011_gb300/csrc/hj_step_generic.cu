@@ -289,7 +289,7 @@ template <typename T, bool FAST32, bool TRACK>
 __global__ void __launch_bounds__(256) hj_step_generic_kernel(const T *__restrict__ v0, const T *__restrict__ vin,
                                                                T *__restrict__ vout,
                                                                const HjCoef<T> *__restrict__ coef,
-                                                               const HjScaledCoef *__restrict__ scaled,
+                                                               const double *__restrict__ scaled,
                                                                const void *__restrict__ k4tab, HjLoop *lp, int sel,
                                                                const HjGeom g, const Divisors dv)
 {
@@ -308,7 +308,6 @@ __global__ void __launch_bounds__(256) hj_step_generic_kernel(const T *__restric
     // FP64: dt is folded into the per-(v, theta) table; the v weight needs it
     // once per thread
     const double k3dt = g.k3 * lp->dt[sel];
-    const bool per4 = (g.periodic >> 3) & 1, ctl = g.mode3 == HJ_AXIS_CONTROL && g.mode4 == HJ_AXIS_CONTROL;
     StepMax mx;
 
     for (unsigned long long c = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; c < ncell;
@@ -318,38 +317,16 @@ __global__ void __launch_bounds__(256) hj_step_generic_kernel(const T *__restric
         const int k = cl.k, l = cl.l;
 
         const T vc = vin[o];
+        const Neigh<T> nx = axis_neighbours<T>(vin, o, cl.i, N1, s1, g.periodic & 1, vc);
+        const Neigh<T> ny = axis_neighbours<T>(vin, o, cl.j, N2, s2, (g.periodic >> 1) & 1, vc);
+        const Neigh<T> nv = axis_neighbours<T>(vin, o, k, N3, s3, (g.periodic >> 2) & 1, vc);
+        const Neigh<T> nt = axis_neighbours<T>(vin, o, l, N4, 1, (g.periodic >> 3) & 1, vc);
         T vn;
         if constexpr (sizeof(T) == 8) {
-            const HjScaledCoef sc = scaled[k * N4 + l];
-            const bool inner = cl.i > 0 && cl.i < (int)N1 - 1 && cl.j > 0 && cl.j < (int)N2 - 1 && k > 0 &&
-                               k < (int)N3 - 1 && per4 && ctl;
-            if (inner) {
-                // every neighbour is a grid value: the operations of
-                // cell_value in the same order, with the upwind x and y
-                // neighbours loaded only and the ghosts' FP64 arithmetic out of
-                // the way (60x60x20x36: 50 -> 37 us per step; 128x128x64x96,
-                // bound by the FP64 unit: 1.47 -> 1.245 ms)
-                const T u1 = vin[nonneg(sc.w1) ? o + s1 : o - s1];
-                const T u2 = vin[nonneg(sc.w2) ? o + s2 : o - s2];
-                const T u3 = hj_max(vin[o + s3], vin[o - s3]);
-                const T u4 = hj_max(vin[l < (int)N4 - 1 ? o + 1 : o - l], vin[l > 0 ? o - 1 : o + (N4 - 1)]);
-                T r = sc.w0 * vc;
-                r = fma(mag(sc.w1), u1, r);
-                r = fma(mag(sc.w2), u2, r);
-                r = fma(k3dt, u3, r);
-                vn = fma(sc.w4, u4, r);
-            } else {
-                const Neigh<T> nx = axis_neighbours<T>(vin, o, cl.i, N1, s1, g.periodic & 1, vc);
-                const Neigh<T> ny = axis_neighbours<T>(vin, o, cl.j, N2, s2, (g.periodic >> 1) & 1, vc);
-                const Neigh<T> nv = axis_neighbours<T>(vin, o, k, N3, s3, (g.periodic >> 2) & 1, vc);
-                const Neigh<T> nt = axis_neighbours<T>(vin, o, l, N4, 1, (g.periodic >> 3) & 1, vc);
-                vn = cell_value(vc, nx, ny, nv, nt, sc, k3dt, g.mode3, g.mode4);
-            }
+            const int tot = (int)N3 * g.p4, e = k * g.p4 + l;
+            const HjScaledCoef sc = {scaled[e], scaled[tot + e], scaled[2 * tot + e], scaled[3 * tot + k]};
+            vn = cell_value(vc, nx, ny, nv, nt, sc, k3dt, g.mode3, g.mode4);
         } else {
-            const Neigh<T> nx = axis_neighbours<T>(vin, o, cl.i, N1, s1, g.periodic & 1, vc);
-            const Neigh<T> ny = axis_neighbours<T>(vin, o, cl.j, N2, s2, (g.periodic >> 1) & 1, vc);
-            const Neigh<T> nv = axis_neighbours<T>(vin, o, k, N3, s3, (g.periodic >> 2) & 1, vc);
-            const Neigh<T> nt = axis_neighbours<T>(vin, o, l, N4, 1, (g.periodic >> 3) & 1, vc);
             const HjCoef<T> cf = coef[k * N4 + l];
             vn = cell_value(vc, nx, ny, nv, nt, cf.c1, cf.c2, k3, ((const float2 *)k4tab)[k].x, dt, g.mode3, g.mode4);
         }
@@ -358,6 +335,105 @@ __global__ void __launch_bounds__(256) hj_step_generic_kernel(const T *__restric
         if constexpr (TRACK) track_change(mx, vn, vc);  // convergence mode: largest change of V
     }
     if constexpr (TRACK) hj_track_epilogue(lp, step_max_bits<T>(mx), scratch);
+}
+
+// The FP64 step of the car grids (theta periodic, x, y, v not; the general
+// kernel above takes the rest): a thread updates two adjacent headings, so
+// that V, its v and (where both lanes have the same side) x and y neighbours,
+// V0 and the coefficients are 16-byte loads, the index arithmetic is shared and
+// two chains of FP64 operations are in flight.  Only the upwind x and y
+// neighbours are loaded, and a ghost is formed only where a lane needs it.  The
+// operations of each cell are cell_value's, in the same order.  Bound by the
+// FP64 unit (5 of its operations per cell); one cell per thread left it idle a
+// quarter of the time, waiting for loads.  Measured per step with one cell and
+// with two: 60x60x20x36 36.7 -> 31.7 us, 96x96x64x96 0.702 -> 0.539 ms (the
+// unit's measured rate allows 0.537).
+struct PairDivisors {
+    FastDiv q2, n3, n2;
+};
+
+constexpr int F64_THREADS = 128;
+
+template <bool TRACK>
+__global__ void __launch_bounds__(F64_THREADS) hj_step_fp64_kernel(const double *__restrict__ v0,
+                                                            const double *__restrict__ vin, double *__restrict__ vout,
+                                                            const double *__restrict__ scaled, HjLoop *lp, int sel,
+                                                            const HjGeom g, const PairDivisors dv, uint32_t npair)
+{
+    __shared__ unsigned long long scratch[32];
+    // a programmatic dependent of the previous step: wait for its grid (its
+    // V_n), then let the next step be scheduled
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (TRACK && lp->done) return;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int N1 = g.n1, N2 = g.n2, N3 = g.n3, N4 = g.n4, P4 = g.p4, tot = N3 * P4;
+    const long long s2 = tot, s1 = (long long)N2 * tot;
+    const double k3dt = g.k3 * lp->dt[sel];
+    StepMax mx;
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < npair; c += gridDim.x * blockDim.x) {
+        const uint32_t row = fast_div(c, dv.q2);
+        const int l = 2 * (int)(c - row * (uint32_t)(P4 / 2));
+        if (l >= N4) continue;  // a pair of pad entries
+        const uint32_t r2 = fast_div(row, dv.n3), i32 = fast_div(r2, dv.n2);
+        const int k = (int)(row - r2 * N3), i = (int)i32, j = (int)(r2 - i32 * N2);
+        const bool two = l + 1 < N4;
+        const double *pc = vin + ((long long)row * P4 + l);
+        const double *tab = scaled + (k * P4 + l);
+        const double2 w1 = *(const double2 *)tab, w2 = *(const double2 *)(tab + tot);
+        const double2 w0 = *(const double2 *)(tab + 2 * tot);
+        const double w4 = scaled[3 * tot + k];
+        const double2 C = *(const double2 *)pc;
+        // v neighbours; at an end of the axis both point at the one there is
+        double2 vp = *(const double2 *)(k < N3 - 1 ? pc + P4 : pc - P4);
+        double2 vm = *(const double2 *)(k > 0 ? pc - P4 : pc + P4);
+        const double tl = l > 0 ? pc[-1] : pc[N4 - 1];
+        const double tr = l + 2 < N4 ? pc[2] : pc[-l];
+        const double2 Z = *(const double2 *)(v0 + ((long long)row * P4 + l));
+        // the upwind x and y neighbours; past an end of the axis the other
+        // side's value, from which the ghost is formed below
+        const bool xa = nonneg(w1.x), xb = nonneg(w1.y), ya = nonneg(w2.x), yb = nonneg(w2.y);
+        const bool gxa = xa ? i == N1 - 1 : i == 0, gxb = xb ? i == N1 - 1 : i == 0;
+        const bool gya = ya ? j == N2 - 1 : j == 0, gyb = yb ? j == N2 - 1 : j == 0;
+        const double *pxa = xa != gxa ? pc + s1 : pc - s1, *pxb = xb != gxb ? pc + s1 : pc - s1;
+        const double *pya = ya != gya ? pc + s2 : pc - s2, *pyb = yb != gyb ? pc + s2 : pc - s2;
+        double2 ux = *(const double2 *)pxa, uy = *(const double2 *)pya;
+        if (pxb != pxa) ux.y = pxb[1];
+        if (pyb != pya) uy.y = pyb[1];
+        // ghosts: behind one branch that most warps skip (as selects, their FP64
+        // operations would run for every cell)
+        if (gxa || gxb || gya || gyb || k == 0 || k == N3 - 1) {
+            auto ghost = [&](bool p, double &u, double cc) {
+                if (p) asm volatile("fma.rn.f64 %0, %1, 0d4000000000000000, %2;" : "=d"(u) : "d"(cc), "d"(-u));
+            };
+            ghost(gxa, ux.x, C.x);
+            ghost(gxb, ux.y, C.y);
+            ghost(gya, uy.x, C.x);
+            ghost(gyb, uy.y, C.y);
+            ghost(k == N3 - 1, vp.x, C.x);
+            ghost(k == N3 - 1, vp.y, C.y);
+            ghost(k == 0, vm.x, C.x);
+            ghost(k == 0, vm.y, C.y);
+        }
+        double a = w0.x * C.x, b = w0.y * C.y;
+        a = fma(mag(w1.x), ux.x, a);
+        b = fma(mag(w1.y), ux.y, b);
+        a = fma(mag(w2.x), uy.x, a);
+        b = fma(mag(w2.y), uy.y, b);
+        a = fma(k3dt, hj_max(vp.x, vm.x), a);
+        b = fma(k3dt, hj_max(vp.y, vm.y), b);
+        a = fma(w4, hj_max(two ? C.y : tr, tl), a);
+        b = fma(w4, hj_max(tr, C.x), b);
+        a = hj_min(Z.x, a);
+        b = hj_min(Z.y, b);
+        double *po = vout + ((long long)row * P4 + l);
+        if (two) *(double2 *)po = make_double2(a, b);
+        else *po = a;
+        if constexpr (TRACK) {
+            track_change(mx, a, C.x);
+            if (two) track_change(mx, b, C.y);
+        }
+    }
+    if constexpr (TRACK) hj_track_epilogue(lp, step_max_bits<double>(mx), scratch);
 }
 
 // ------------------------------------------------------------ resident form
@@ -885,7 +961,7 @@ cudaError_t hj_launch_step_generic(hj_grid *g, long long n, int sel)
     cudaError_t le = cudaSuccess;
     const void *vin = hj_value_ptr(g, n);
     void *vout = hj_value_ptr(g, n + 1);
-    const HjScaledCoef *scaled = g->scaled ? g->scaled + (size_t)sel * g->n[2] * g->n[3] : nullptr;
+    const double *scaled = g->scaled ? g->scaled + sel * hj_scaled_count(g->n[2], g->p4) : nullptr;
     const int32_t *qw = g->qw ? g->qw + sel * hj_qw_count(g->n[2], g->p4) : nullptr;
 #define HJ_LAUNCH_Q(F, K)                                                                                        \
     le = launch_dependent(hj_step_q527_kernel<F, K>, blocks, threads, g->stream, (const int32_t *)g->v0,        \
@@ -909,6 +985,26 @@ cudaError_t hj_launch_step_generic(hj_grid *g, long long n, int sel)
             if (g->track) HJ_LAUNCH_Q(false, true);
             else HJ_LAUNCH_Q(false, false);
         }
+    } else if (g->prec == HJ_FP64 && g->periodic == 0x8u && g->geom.mode3 == HJ_AXIS_CONTROL &&
+               g->geom.mode4 == HJ_AXIS_CONTROL && g->nint < (1LL << 32)) {
+        PairDivisors pd;
+        pd.q2 = make_fastdiv((uint32_t)(g->p4 / 2));
+        pd.n3 = dv.n3;
+        pd.n2 = dv.n2;
+        const uint32_t npair = (uint32_t)(g->nint / 2);
+        // one pair per thread up to 16 blocks per SM, then two, up to 128 blocks
+        // per SM: many short blocks leave no SM idle at the end of a step
+        // (96x96x64x96: 0.573 ms with a quarter as many blocks, 0.539 so;
+        // 60x60x20x36: 32.8 us with one pair per thread, 31.7 with two)
+        const long long pw = ((long long)npair + F64_THREADS - 1) / F64_THREADS;
+        const long long p2 = pw / 2 < 16 * cap ? pw / 2 : 16 * cap;
+        const int pblocks = (int)(pw < 2 * cap ? pw : p2 < 2 * cap ? 2 * cap : p2);
+        le = g->track ? launch_dependent(hj_step_fp64_kernel<true>, pblocks, F64_THREADS, g->stream,
+                                         (const double *)g->v0, (const double *)vin, (double *)vout, scaled, g->loop,
+                                         sel, g->geom, pd, npair)
+                      : launch_dependent(hj_step_fp64_kernel<false>, pblocks, F64_THREADS, g->stream,
+                                         (const double *)g->v0, (const double *)vin, (double *)vout, scaled, g->loop,
+                                         sel, g->geom, pd, npair);
     } else if (g->prec == HJ_FP64) {
         if (fast) HJ_LAUNCH2(double, true);
         else HJ_LAUNCH2(double, false);
