@@ -52,6 +52,8 @@ constexpr int B_VARIANTS[4] = {352, 480, 608, 736};
 constexpr int B_DUAL = 288;
 // Batch steps (rounds) per launch at most.
 constexpr int B_MAX_ROUNDS = 1024;
+// Memory of removed slots a batch keeps at most.
+constexpr size_t B_POOL_BYTES = 1ull << 30;
 
 struct BatchInst {
     int n1, n2, n3, n4, p4, q4;
@@ -637,6 +639,11 @@ struct SlotHost {
 struct hj_batch {
     int max_slots = 0;
     size_t budget = 0, used_bytes = 0;
+    // device memory of removed slots, kept for the next ones of the same size (a
+    // served request costs an allocation and a free otherwise): at most
+    // B_POOL_BYTES, and within the budget together with the slots in use
+    std::vector<std::pair<void *, size_t>> pool;
+    size_t pool_bytes = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int device = 0, sms = 0, maxsmem = 0, smem_sm = 0;
@@ -657,6 +664,7 @@ struct hj_batch {
     BatchParams bp = {0, 0, 0};
     int ctas = 0;
     bool dirty = true;
+    bool fresh = false;  // h_slots' states are the device's (nothing queued since they were read)
     int *d_rounds = nullptr;       // queue position of each round of a launch (B_MAX_ROUNDS + 1)
     int *d_rounds_done = nullptr;  // per slot: steps finalised in the current launch
     std::vector<int> h_rounds;     // source of the stream-ordered copy into d_rounds
@@ -692,6 +700,44 @@ hj_status bfail(hj_status s, const char *fmt, ...)
         }                                                                                                \
     } while (0)
 
+
+void release_pool(hj_batch *b)
+{
+    for (auto &m : b->pool) cudaFree(m.first);
+    b->pool.clear();
+    b->pool_bytes = 0;
+}
+
+// Device memory of a new slot: a kept block of that size, else a fresh one.
+cudaError_t slot_alloc(hj_batch *b, size_t bytes, void **mem)
+{
+    for (size_t i = 0; i < b->pool.size(); ++i)
+        if (b->pool[i].second == bytes) {
+            *mem = b->pool[i].first;
+            b->pool_bytes -= bytes;
+            b->pool.erase(b->pool.begin() + i);
+            return cudaSuccess;
+        }
+    if (b->used_bytes + b->pool_bytes + bytes > b->budget) release_pool(b);
+    cudaError_t e = cudaMalloc(mem, bytes);
+    if (e == cudaErrorMemoryAllocation && !b->pool.empty()) {
+        cudaGetLastError();
+        release_pool(b);
+        e = cudaMalloc(mem, bytes);
+    }
+    return e;
+}
+
+// Memory of a removed slot (no longer in used_bytes; the stream is idle).
+void slot_free(hj_batch *b, void *mem, size_t bytes)
+{
+    if (b->used_bytes + b->pool_bytes + bytes > b->budget || b->pool_bytes + bytes > B_POOL_BYTES) {
+        cudaFree(mem);
+        return;
+    }
+    b->pool.push_back({mem, bytes});
+    b->pool_bytes += bytes;
+}
 
 // Tile of one slot for a block of nc consumer threads (ty x tv <= nc / q4).
 // Every item costs the whole block a pass over its planes, whether its rows
@@ -819,17 +865,12 @@ hj_status rebuild(hj_batch *b)
 {
     BEncodeFn enc = batch_encode_fn();
     if (!enc) return bfail(HJ_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
-    // block size: the request, else the smallest variant that gives every
-    // slot at least 32 rows
-    int nc = b->nconsumer_req;
-    if (nc <= 0) {
-        nc = B_VARIANTS[0];
-        for (auto &s : b->slots)
-            if (s.used) {
-                const int need = (s.p4 / 4) * 32;
-                while (nc < need && nc < B_VARIANTS[3]) nc += 128;
-            }
-    }
+    // block size: the request, else 480 consumers.  Device ms of whole solves with
+    // 288 (two CTAs per SM), 352 and 480 consumers: 64 slots of up to 60x60x24x36
+    // 19.4, 22.8, 19.7; 16 of them 6.1, 6.3, 5.5; 4 of them 2.27, 2.23, 2.38; eight
+    // of 31x31x11x16 to 100x100x30x48 5.3, 5.7, 4.9; one of 128x128x64x96 (18 steps)
+    // 4.3, 4.0, 3.6.
+    const int nc = b->nconsumer_req > 0 ? b->nconsumer_req : B_VARIANTS[1];
     b->h_insts.assign(b->max_slots, BatchInst());
     std::vector<BatchInst> &insts = b->h_insts;
     std::vector<CUtensorMap> maps((size_t)4 * b->max_slots);
@@ -992,6 +1033,7 @@ hj_status run_rounds(hj_batch *b, const std::vector<long long> &ki, long long k)
     b->lay_nitems = (int)pos;
     HJB_CUDA(cudaMemcpyAsync((char *)b->d_ctl + offsetof(BatchCtl, nitems), &b->lay_nitems, sizeof(int),
                              cudaMemcpyHostToDevice, b->stream));
+    b->fresh = false;
     BatchKernelFn fn = batch_kernel(b->bp.nconsumer);
     fn<<<b->ctas, b->bp.nconsumer + 32, batch_smem(b->bp), b->stream>>>(b->d_insts, b->d_slots, b->d_items, b->d_ctl,
                                                                         b->d_maps, b->bp, b->d_rounds,
@@ -1024,11 +1066,13 @@ hj_status pull_slots(hj_batch *b)
     HJB_CUDA(cudaMemcpyAsync(b->h_slots, b->d_slots, sizeof(BatchSlot) * b->max_slots, cudaMemcpyDeviceToHost,
                              b->stream));
     HJB_CUDA(cudaStreamSynchronize(b->stream));
+    b->fresh = true;
     return HJ_OK;
 }
 
 hj_status push_slot(hj_batch *b, int i)
 {
+    b->fresh = false;
     HJB_CUDA(cudaMemcpyAsync(&b->d_slots[i], &b->h_slots[i], sizeof(BatchSlot), cudaMemcpyHostToDevice, b->stream));
     HJB_CUDA(cudaStreamSynchronize(b->stream));
     return HJ_OK;
@@ -1039,6 +1083,7 @@ hj_status push_slot(hj_batch *b, int i)
 // mirror entry is not written again before then.
 hj_status push_slot_async(hj_batch *b, int i)
 {
+    b->fresh = false;
     HJB_CUDA(cudaMemcpyAsync(&b->d_slots[i], &b->h_slots[i], sizeof(BatchSlot), cudaMemcpyHostToDevice, b->stream));
     return HJ_OK;
 }
@@ -1125,6 +1170,7 @@ void hj_batch_destroy(hj_batch *b)
     if (b->stream) cudaStreamSynchronize(b->stream);
     for (auto &s : b->slots)
         if (s.mem) cudaFree(s.mem);
+    release_pool(b);
     if (b->d_insts) cudaFree(b->d_insts);
     if (b->d_slots) cudaFree(b->d_slots);
     if (b->h_slots) cudaFreeHost(b->h_slots);
@@ -1211,7 +1257,7 @@ hj_status hj_batch_add(hj_batch *b, const int32_t n[4], const double lo[4], cons
     s.p4 = p4;
     s.nint = nint;
     s.ncell = (long long)n[0] * n[1] * n[2] * n[3];
-    HJB_CUDA(cudaMalloc(&s.mem, bytes));
+    HJB_CUDA(slot_alloc(b, bytes, &s.mem));
     s.bytes = bytes;
     size_t sz_v0, sz_ab, sz_coef, sz_tab, sz_amax;
     slot_layout(n, &sz_v0, &sz_ab, &sz_coef, &sz_tab, &sz_amax);
@@ -1237,7 +1283,7 @@ hj_status hj_batch_add(hj_batch *b, const int32_t n[4], const double lo[4], cons
     b->slots[slot] = s;
     hj_status st = upload_slot_tables(b, b->slots[slot]);
     if (st != HJ_OK) {
-        cudaFree(s.mem);
+        slot_free(b, s.mem, s.bytes);
         b->slots[slot] = SlotHost();
         return st;
     }
@@ -1259,8 +1305,8 @@ hj_status hj_batch_remove(hj_batch *b, int32_t slot)
     memset(&b->h_slots[slot], 0, sizeof(BatchSlot));
     b->h_slots[slot].st.done = 1;
     if ((s = push_slot(b, slot)) != HJ_OK) return s;
-    cudaFree(b->slots[slot].mem);
     b->used_bytes -= b->slots[slot].bytes;
+    slot_free(b, b->slots[slot].mem, b->slots[slot].bytes);
     b->slots[slot] = SlotHost();
     b->dirty = true;
     return HJ_OK;
@@ -1382,6 +1428,7 @@ hj_status hj_batch_set_initial_values_device(hj_batch *b, int32_t nslots, const 
         if ((s = ingest_check(b, slots[k], v0[k], counts[k])) != HJ_OK) return s;
     if (nslots == 0) return HJ_OK;
     if ((s = order_after_default_stream(b)) != HJ_OK) return s;
+    b->fresh = false;
     // reset the slots' states: the mirror entries, pushed as runs of
     // consecutive slots
     for (int32_t k = 0; k < nslots; ++k) {
@@ -1443,6 +1490,7 @@ hj_status hj_batch_set_horizon(hj_batch *b, int32_t slot, double T, double cfl)
     if (!sl.has_value) return bfail(HJ_ERR_STATE, "slot %d has no initial value", slot);
     sl.T = T;
     sl.cfl = cfl;
+    b->fresh = false;
     // queued on the batch's stream (ordered before the next batch step); the
     // calls that read slot states synchronise first
     HJB_CUDA(hj_launch_prologue_f32(&b->d_slots[slot].st, sl.geom, sl.coef, sl.n[2] * sl.n[3], T, cfl, b->stream));
@@ -1464,6 +1512,7 @@ hj_status hj_batch_set_horizons(hj_batch *b, int32_t nslots, const int32_t *slot
         if (!b->slots[slots[k]].has_value) return bfail(HJ_ERR_STATE, "slot %d has no initial value", slots[k]);
     }
     if (nslots == 0) return HJ_OK;
+    b->fresh = false;
     HJB_CUDA(cudaEventSynchronize(b->ev_setup));  // the previous list has been copied
     for (int32_t k = 0; k < nslots; ++k) {
         SlotHost &sl = b->slots[slots[k]];
@@ -1575,7 +1624,7 @@ static hj_status batch_read(hj_batch *b, int32_t slot, void *out, hj_precision d
     if (!out) return bfail(HJ_ERR_INVALID_ARG, "out is NULL");
     if (count != (size_t)sl.ncell) return bfail(HJ_ERR_INVALID_ARG, "count %zu != %lld", count, sl.ncell);
     if (!sl.has_value) return bfail(HJ_ERR_STATE, "slot %d has no initial value", slot);
-    if ((s = pull_slots(b)) != HJ_OK) return s;
+    if (!b->fresh && (s = pull_slots(b)) != HJ_OK) return s;
     const long long n = b->h_slots[slot].st.n;
     const float *src = n == 0 ? sl.v0 : sl.buf + ((n - 1) & 1) * sl.nint;
     const long long nrows = (long long)sl.n[0] * sl.n[1] * sl.n[2];
@@ -1640,6 +1689,7 @@ hj_status hj_batch_autotune(hj_batch *b, int32_t steps_per_trial, int32_t *best_
     for (int i = 0; i < b->max_slots; ++i)
         if (b->slots[i].used && (b->h_slots[i].st.n != 0 || !b->slots[i].has_value))
             return bfail(HJ_ERR_STATE, "autotune needs every slot right after its initial value (slot %d)", i);
+    b->fresh = false;
     std::vector<BatchSlot> saved(b->h_slots, b->h_slots + b->max_slots);
     const int keep_nc = b->nconsumer_req, keep_ch = b->xc_mode;
     double best = 1e300;
