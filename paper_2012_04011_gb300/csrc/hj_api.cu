@@ -62,13 +62,15 @@ __device__ __forceinline__ T elem_from_f64(double x)
 }
 
 // Dense row-major [N1][N2][N3][N4] (any of double/float) -> internal layout
-// (rows padded to p4, pad lanes zero).  Flags non-finite input.
+// (rows padded to p4, pad lanes zero).  Flags non-finite input.  With nonflat
+// given, also flags a value that differs from the first one of its column (n3
+// rows) and stores those first values in xy.
 template <typename Tin, typename T>
 __global__ void ingest_kernel(const Tin *__restrict__ src, T *__restrict__ dst, int n4, int p4, long long nrows,
-                              int *nonfinite)
+                              int *nonfinite, int *nonflat = nullptr, int n3 = 1, T *xy = nullptr)
 {
     long long total = nrows * p4;
-    int bad = 0;
+    int bad = 0, varies = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
         long long row = i / p4;
@@ -78,10 +80,17 @@ __global__ void ingest_kernel(const Tin *__restrict__ src, T *__restrict__ dst, 
             double x = elem_to_f64<Tin>(src[row * n4 + l]);
             if (!isfinite(x)) bad = 1;
             v = elem_from_f64<T>(x);
+            if (nonflat) {  // (the sign of a zero counts)
+                const long long col = row / n3;
+                const T first = elem_from_f64<T>(elem_to_f64<Tin>(src[col * n3 * n4]));
+                if (v != first || signbit((double)v) != signbit((double)first)) varies = 1;
+                if (l == 0 && row == col * n3) xy[col] = v;
+            }
         }
         dst[i] = v;
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0) *(volatile int *)nonfinite = 1;
+    if (nonflat && __syncthreads_or(varies) && threadIdx.x == 0) *(volatile int *)nonflat = 1;
 }
 
 // V0 that depends only on (x, y): an N1*N2 field replicated over v and theta
@@ -316,6 +325,7 @@ void reset_state(hj_grid *g)
     g->nstep = 0;
     g->hflags->status = HJ_OK;
     g->hflags->nonfinite = 0;
+    g->hflags->nonflat = 0;
 }
 
 // Whether HJ_KERNEL_AUTO takes the resident kernel: FP32 grids of up to 4 M
@@ -718,6 +728,19 @@ static void set_v0_mode(hj_grid *g, bool bcast)
     }
 }
 
+// Whether a 4D V0 is worth checking for one value per (x, y), which any V0 of
+// Eq. init_V has (it depends on the position only): the ingest reads every
+// value anyway, and the tiled kernel then reads the field instead of V0 boxes,
+// 8 instead of 12 bytes of memory traffic per cell-update, same bits.  It pays
+// on FP32 grids that stream from memory and take the single-sided form: us per
+// step with V0 boxes and with the field, autotuned, 96x96x32x64 38.1 and 29.5,
+// 128x128x64x96 179 and 130.  The general form gains nothing (127x119x61x93 165
+// and 169), nor does a grid that stays in L2 (80x80x25x40 14.6 and 14.6).
+static bool check_flat(const hj_grid *g)
+{
+    return g->prec == HJ_FP32 && g->tiled_ok && g->tiled_usign && g->p4 == g->n[3] && g->ncell >= (1LL << 24);
+}
+
 static hj_status finish_ingest(hj_grid *g);
 
 // V0 from its (x, y) field on the device (src: nxy values of dtype): the 4D
@@ -737,8 +760,29 @@ static hj_status ingest_xy(hj_grid *g, const void *src, hj_precision dtype, long
                                                                                 (int)nxy, (int)nxy, 1, flag);
         });
     });
+    g->v0_xy = true;
     set_v0_mode(g, true);
     return finish_ingest(g);
+}
+
+// V0 from a dense 4D array the device can read.
+static hj_status ingest_4d(hj_grid *g, const void *src, hj_precision dtype)
+{
+    const long long nrows = (long long)g->n[0] * g->n[1] * g->n[2];
+    const bool check = check_flat(g);
+    with_elem(dtype, [&](auto ein) {
+        with_elem(g->prec, [&](auto e) {
+            using Tin = decltype(ein);
+            using T = decltype(e);
+            ingest_kernel<Tin, T><<<grid_blocks(g->nint, 256), 256, 0, g->stream>>>(
+                (const Tin *)src, (T *)g->v0, g->n[3], g->p4, nrows, &g->dflags->nonfinite,
+                check ? &g->dflags->nonflat : nullptr, g->n[2], (T *)g->v0xy);
+        });
+    });
+    g->v0_xy = false;
+    const hj_status s = finish_ingest(g);
+    set_v0_mode(g, s == HJ_OK && check && !*(volatile int *)&g->hflags->nonflat);
+    return s;
 }
 
 static hj_status finish_ingest(hj_grid *g)
@@ -798,15 +842,7 @@ hj_status hj_set_initial_value(hj_grid *g, const double *v0, size_t count)
         staging = (const double *)g->buf;
         HJ_CUDA(cudaMemcpyAsync(g->buf, v0, sizeof(double) * (size_t)g->ncell, cudaMemcpyHostToDevice, g->stream));
     }
-    long long nrows = (long long)g->n[0] * g->n[1] * g->n[2];
-    int *flag = &g->dflags->nonfinite;
-    int blocks = grid_blocks(g->nint, 256);
-    with_elem(g->prec, [&](auto e) {
-        using T = decltype(e);
-        ingest_kernel<double, T><<<blocks, 256, 0, g->stream>>>(staging, (T *)g->v0, g->n[3], g->p4, nrows, flag);
-    });
-    set_v0_mode(g, false);
-    return finish_ingest(g);
+    return ingest_4d(g, staging, HJ_FP64);
 }
 
 hj_status hj_set_initial_value_xy(hj_grid *g, const double *v0_xy, size_t count)
@@ -851,19 +887,7 @@ hj_status hj_set_initial_value_device(hj_grid *g, const void *v0_device, hj_prec
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;
     reset_state(g);
-    long long nrows = (long long)g->n[0] * g->n[1] * g->n[2];
-    int *flag = &g->dflags->nonfinite;
-    int blocks = grid_blocks(g->nint, 256);
-    with_elem(dtype, [&](auto ein) {
-        with_elem(g->prec, [&](auto e) {
-            using Tin = decltype(ein);
-            using T = decltype(e);
-            ingest_kernel<Tin, T><<<blocks, 256, 0, g->stream>>>((const Tin *)v0_device, (T *)g->v0, g->n[3], g->p4,
-                                                                 nrows, flag);
-        });
-    });
-    set_v0_mode(g, false);
-    return finish_ingest(g);
+    return ingest_4d(g, v0_device, dtype);
 }
 
 // The time loop of hj_advance_brt and hj_solve_converged (threshold > 0:
@@ -1368,7 +1392,7 @@ hj_status hj_get_info(const hj_grid *g, hj_grid_info *info)
     }
     info->pitch4 = g->p4;
     info->precision = g->prec;
-    info->v0_broadcast = g->v0_bcast ? 1 : 0;
+    info->v0_broadcast = g->v0_xy ? 1 : 0;
     info->kernel = effective_kernel(g);
     info->periodic_mask = g->periodic;
     info->has_value = g->has_value;

@@ -56,6 +56,7 @@ struct HjLoop {
 struct HjFlags {
     int status;     // hj_status raised on the device (HJ_OK if none)
     int nonfinite;  // an ingest saw a NaN or Inf
+    int nonflat;    // an ingest saw a V0 that varies within a column (one (x, y))
 };
 
 // FP64 coefficients with dt folded in (per (v, theta)): w1 = dt xdot_1/dx_1,
@@ -124,7 +125,9 @@ struct hj_grid {
     void *k4tab;           // theta coefficient per speed: |xdot_4|/dx_4 (double[n3]; FP32 grids: float2[n3] of
                            // (k4, -(k3 + k4)))
     void *v0xy;            // V0 as an N1 x N2 field (element type of the grid), when V0 depends on x, y only
-    bool v0_bcast;         // V0 was set from the (x, y) field: the tiled kernel reads v0xy
+    bool v0_xy;            // V0 was set from the (x, y) field
+    bool v0_bcast;         // the tiled kernel reads V0 from v0xy: it was set from the field, or a 4D V0 turned
+                           // out to have one value per (x, y) on a grid where that form is the faster one
     bool track;            // a convergence-mode call is running: launch the kernels that reduce the change
     float *tab_tiled;      // tiled-kernel tables: v_k [n3], cos/dx1 [p4], sin/dx2 [p4], quad signs [p4]
     HjLoop *loop;          // device constants of the current solve call

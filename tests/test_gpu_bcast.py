@@ -154,3 +154,32 @@ def test_broadcast_v0_full_size_same_bits(hj):
             g.read_value_device(out)
             outs.append(out.cpu().numpy())
     assert np.array_equal(outs[0], outs[1])
+
+
+def test_flat_4d_v0_is_recognised_and_one_odd_cell_is_not_lost(hj):
+    """A 4D V0 with one value per (x, y) on a grid of 2^24 cells takes the field
+    form of the tiled kernel (same bits as the field itself); with a single cell
+    changed it must not: that cell keeps its own V0, and away from it nothing
+    changes."""
+    w = scenes.custom_workload((64, 64, 64, 64), n_circles=4, T=0.1, seed=5)
+    V0 = scenes.initial_value(w.grid, w.scene).astype(np.float32)
+    import torch
+    outs = []
+    odd = V0.copy()
+    cell = (30, 20, 40, 50)
+    odd[cell] -= 0.5
+    for v0, xy in ((None, True), (V0, False), (odd, False)):
+        with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+            if xy:
+                g.set_initial_value_xy(scenes.signed_distance_xy(w.grid, w.scene))
+            else:
+                g.set_initial_value(torch.from_numpy(v0).cuda())
+            assert g.info().v0_broadcast == int(xy)
+            g.advance_brt(w.T, w.cfl, 3)
+            out = torch.empty(V0.shape, dtype=torch.float32, device="cuda")
+            outs.append(g.read_value_device(out).cpu().numpy())
+    assert np.array_equal(outs[0], outs[1])
+    assert outs[2][cell] <= odd[cell] < outs[1][cell]
+    far = np.ones(V0.shape, bool)
+    far[27:34, 17:24, 37:44, 47:54] = False  # three steps reach three cells
+    assert np.array_equal(outs[2][far], outs[1][far])

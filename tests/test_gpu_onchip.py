@@ -60,6 +60,6 @@ def test_onchip_equals_generic(hj, n, prec, flat):
     V0 = scenes.initial_value(w.grid, w.scene) if flat else smooth_v0(n, sum(n))
     for steer, lo in ((False, scenes.DOMAIN_LO), (True, (-5.0, -5.0, -2.0, -np.pi))):
         ref, steps = solve(hj, n, code, hj.HJ_KERNEL_GENERIC, V0, steer, lo=lo)
-        for chunk in (None, 3):
+        for chunk in (None, 2, 3):
             got, s2 = solve(hj, n, code, hj.HJ_KERNEL_RESIDENT, V0, steer, chunk, lo)
             assert s2 == steps and np.array_equal(got, ref), (steer, chunk)
