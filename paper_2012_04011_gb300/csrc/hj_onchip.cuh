@@ -114,6 +114,8 @@ __device__ __forceinline__ bool wait_published(const unsigned int *p, unsigned i
 // What a thread knows about its quad for the whole launch.
 struct Thread {
     float K1[4], K2[4], k3, k4;  // FP32: |xdot_d| / dx_d; Q5.27: weight magnitudes (int32 bits)
+    int32_t nsum[4];             // Q5.27: -(sum of the four weights)
+    bool wsmall;                 // Q5.27: none below -2^30 (hj_q527_update_interior32)
     uint32_t mx[4], my[4];
     uint32_t sx;
     int ovm, ovp, lidx, ridx, lreal, cs;
@@ -204,32 +206,39 @@ __device__ __forceinline__ void sweep(const Thread &T, SweepIO io, const float d
             if (gyp) yb = ym;
             const bool anyg = T.gvm || T.gvp || (T.xmix ? (T.gxm || T.gxp) : T.gu) || gym || gyp;
             const int32_t w3 = fi(T.k3), w4 = fi(T.k4);
+            int32_t tt[4];  // the larger theta neighbour
+            tt[0] = max(fi(PADDED && lreal == 1 ? tr : c.y), fi(tl));
+            tt[1] = max(fi(PADDED && lreal == 2 ? tr : c.z), fi(c.x));
+            tt[2] = max(fi(PADDED && lreal == 3 ? tr : c.w), fi(c.y));
+            tt[3] = max(fi(tr), fi(c.z));
+            if (!anyg && T.wsmall) {  // every neighbour is a grid value
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const bool xpos = (T.sx >> e) & 1u;
-                const int32_t vc = fi(f4get(c, e)), a1 = fi(T.K1[e]), a2 = fi(T.K2[e]);
-                const int32_t tm = fi(e == 0 ? tl : f4get(c, e > 0 ? e - 1 : 0));
-                int32_t tp = fi(e == 3 ? tr : f4get(c, e < 3 ? e + 1 : 3));
-                if (PADDED && e < 3 && e == lreal - 1) tp = fi(tr);
-                const int32_t nsum = -(a1 + a2 + w3 + w4);
-                const int32_t za = fi(f4get(z, e));
-                const int32_t u1 = fi(MIX ? bitsel(T.mx[e], f4get(xb, e), f4get(xa, e)) : f4get(ux, e));
-                const int32_t u2 = fi(bitsel(T.my[e], f4get(yb, e), f4get(ya, e)));
-                const int32_t pv = fi(f4get(vp, e)), mv = fi(f4get(vm, e)), u3 = max(pv, mv);
-                int32_t vn;
-                if (!anyg && nsum >= -(1 << 30)) {
-                    vn = hj_q527_update_interior32(vc, za, u1, u2, u3, max(tp, tm), a1, a2, w3, w4, nsum);
-                } else {
+                for (int e = 0; e < 4; ++e) {
+                    const int32_t u1 = fi(MIX ? bitsel(T.mx[e], f4get(xb, e), f4get(xa, e)) : f4get(ux, e));
+                    const int32_t u2 = fi(bitsel(T.my[e], f4get(yb, e), f4get(ya, e)));
+                    const int32_t u3 = max(fi(f4get(vp, e)), fi(f4get(vm, e)));
+                    f4set(out, e,
+                          fl(hj_q527_update_interior32(fi(f4get(c, e)), fi(f4get(z, e)), u1, u2, u3, tt[e],
+                                                       fi(T.K1[e]), fi(T.K2[e]), w3, w4, T.nsum[e])));
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const bool xpos = (T.sx >> e) & 1u;
+                    const int32_t vc = fi(f4get(c, e)), a1 = fi(T.K1[e]), a2 = fi(T.K2[e]);
+                    const int32_t u1 = fi(MIX ? bitsel(T.mx[e], f4get(xb, e), f4get(xa, e)) : f4get(ux, e));
+                    const int32_t u2 = fi(bitsel(T.my[e], f4get(yb, e), f4get(ya, e)));
+                    const int32_t pv = fi(f4get(vp, e)), mv = fi(f4get(vm, e)), u3 = max(pv, mv);
                     const bool hxg = T.xmix ? (xpos ? T.gxp : T.gxm) : T.gu;
                     const bool hyg = T.my[e] ? gyp : gym;
                     // v: at an end both pv and mv hold the one grid neighbour o; the larger of o and
                     // its ghost 2 V_c - o (upper end: the ghost if equal, it is V(v + 1))
                     const bool hv = T.gvp ? vc >= mv : (T.gvm ? pv < vc : false);
-                    const int32_t c0 = nsum + (hxg ? 2 * a1 : 0) + (hyg ? 2 * a2 : 0) + (hv ? 2 * w3 : 0);
-                    vn = hj_q527_update_interior(vc, za, u1, u2, u3, max(tp, tm), hxg ? -a1 : a1, hyg ? -a2 : a2,
-                                                 hv ? -w3 : w3, w4, c0);
+                    const int32_t c0 = T.nsum[e] + (hxg ? 2 * a1 : 0) + (hyg ? 2 * a2 : 0) + (hv ? 2 * w3 : 0);
+                    f4set(out, e,
+                          fl(hj_q527_update_interior(vc, fi(f4get(z, e)), u1, u2, u3, tt[e], hxg ? -a1 : a1,
+                                                     hyg ? -a2 : a2, hv ? -w3 : w3, w4, c0)));
                 }
-                f4set(out, e, fl(vn));
             }
         }
         if (PADDED) {  // pad lanes hold 0
@@ -289,13 +298,17 @@ __global__ void __launch_bounds__(MAXT, 1)
         const int32_t *w = FIXED ? qw + (size_t)sel * hj_qw_count(N3, P4) : nullptr;
         T.k3 = FIXED ? fl(w[2 * cs]) : P.k3;
         T.k4 = FIXED ? fl(w[2 * cs + HJ_QW_TAIL + k]) : ((const float2 *)k4tab)[k].x;
+        T.wsmall = true;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
+            T.nsum[e] = 0;
             T.K1[e] = T.K2[e] = 0.f;
             if (e >= lreal) continue;
             if constexpr (FIXED) {
                 T.K1[e] = fl(abs(w[e0 + e]));
                 T.K2[e] = fl(abs(w[cs + e0 + e]));
+                T.nsum[e] = -(fi(T.K1[e]) + fi(T.K2[e]) + fi(T.k3) + fi(T.k4));
+                T.wsmall = T.wsmall && T.nsum[e] >= -(1 << 30);
             } else {
                 const HjCoef<float> c = ((const HjCoef<float> *)coefp)[k * N4 + 4 * q + e];
                 T.K1[e] = fabsf(c.c1);
