@@ -100,6 +100,78 @@ int best_chunk(const hj_grid *g, int ncol, int slots)
     return best_xc;
 }
 
+// Fixed point: the most planes any of the n CTAs sweeps in a step, in planes of
+// an inner tile.  A plane of a tile at an end of v takes 1.7 + 0.5 / tv times as
+// long (extrapolated ghosts take the 64-bit form), at an end of y 1.1 times; the
+// CTAs take the items in next_item()'s order.  Beyond 16 rounds the CTAs' shares
+// are close to the mean, which is used instead.
+double heaviest_q527(const hj_grid *g, const TiledParams &P, int xc, int nchunk, int n)
+{
+    const long long items = (long long)P.ncol * nchunk;
+    double load[1024] = {0.0};
+    const bool mean = items > 16LL * n || n > 1024;
+    if (n > items) n = (int)items;
+    const int ncol_y = P.ncol / P.ncol_v;
+    double sum = 0.0, most = 0.0;
+    int shift = 0, place = 0;
+    for (int c = 0; c < nchunk; ++c) {
+        const int x0 = c * xc, x1 = x0 + xc < g->n[0] ? x0 + xc : g->n[0];
+        const int planes = (x1 < g->n[0] ? x1 + 1 : x1) - (x0 > 0 ? x0 - 1 : 0);
+        for (int col = 0; col < P.ncol; ++col) {
+            const int iv = col % P.ncol_v, iy = col / P.ncol_v;
+            const bool end_v = iv == 0 || iv == P.ncol_v - 1, end_y = iy == 0 || iy == ncol_y - 1;
+            const double w = planes * (end_v ? 1.7 + 0.5 / P.tv : end_y ? 1.1 : 1.0);
+            sum += w;
+            if (!mean) most = fmax(most, load[(place + n - shift) % n] += w);
+            if (++place == n) {
+                place = 0;
+                shift = (shift + 1) % n;
+            }
+        }
+        if (mean && c == 2 && nchunk > 4) {  // the inner chunks are alike
+            sum *= (double)nchunk / 3;
+            break;
+        }
+    }
+    return mean ? sum / n : most;
+}
+
+// Estimated time of a step (in us, up to what all shapes of a grid share) for
+// the default tile: (rounds of items) x (planes one item loads) x (time of a
+// plane).  A plane costs a fixed part (the waits on its stage and the release)
+// and a part per consumer warp that depends on the launch-bound class, which
+// sets the registers; the forms that read V0 as a field also pay for the bytes
+// through shared memory.  Below 8 warps an SM is latency-bound and a plane
+// takes as long as with 8.  In fixed point the tiles' costs differ and the CTA
+// with the heaviest items sets the time.  Coefficients: least squares over the
+// 20 to 40 shapes that hj_autotune timed on each of 10 grids (2 to 101 M
+// cells; in fixed point 18, of which 4 were not in the fit).  Against the best
+// timed shape of each grid the picks take 1.00 to 1.03 times as long with a 4D
+// V0, 1.00 to 1.26 (mean 1.04) with the field and 1.00 to 1.11 (1.02) in fixed
+// point; the shape with the fewest halo reads per row, the rule before, took
+// 1.00 to 1.33 (1.13), 1.03 to 1.26 (1.16) and 1.00 to 1.74 (1.22).  Per step:
+// 80x80x25x40 FP32 18.4 -> 15.4 us, 128x128x64x96 with the field 156 -> 141,
+// 64x64x24x36 Q5.27 35.0 -> 16.0, 100x100x30x48 Q5.27 69.5 -> 55.2,
+// 113x97x47x59 Q5.27 156 -> 109.
+double step_cost(const hj_grid *g, const TiledParams &P, int slots, int xc_req)
+{
+    static const double F4D[4] = {0.0089, 0.0111, 0.0148, 0.0210}, FXY[4] = {0.0169, 0.0147, 0.0176, 0.0209},
+                        Q[4] = {0.0326, 0.0300, 0.0296, 0.0357};
+    const bool fixed = g->prec == HJ_Q527;
+    const int xc = xc_req > 0 && xc_req < g->n[0] ? xc_req : (xc_req > 0 ? g->n[0] : best_chunk(g, P.ncol, slots));
+    const int nchunk = (g->n[0] + xc - 1) / xc;
+    int cls = 0;
+    while (cls < 3 && P.nconsumer > hj_tiled_variant(fixed, cls)) ++cls;
+    const double warps = P.nconsumer > 256 ? P.nconsumer / 32 : 8;
+    const long long rounds = ((long long)P.ncol * nchunk + slots - 1) / slots;
+    const double planes = (double)rounds * (xc + (nchunk > 1 ? 2 : 1));
+    if (fixed) return heaviest_q527(g, P, xc, nchunk, slots) * warps * Q[cls] + planes * 0.25;
+    if (!g->v0_bcast) return planes * (warps * F4D[cls] + 0.2875);
+    const double per_warp = P.rpt == 1 ? FXY[cls] : (P.rpt == 2 ? 2 * 0.0204 : 4 * 0.0152);
+    const double kb = (P.halo_box + g->p4 * P.ty * P.tv) / 256.0;
+    return planes * (warps * per_warp + 0.00497 * kb + 0.1425);
+}
+
 size_t tiled_smem_bytes(const TiledParams &P)
 {
     return (size_t)P.stages * P.stage_bytes + 2 * MAX_STAGES * sizeof(uint64_t) + 32 * sizeof(unsigned long long) +
@@ -187,34 +259,29 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
     if (e != cudaSuccess) return fail("sign table upload failed");
     g->tiled_usign = usign;  // a property of the grid's v and theta ranges (read by tiled_rpt)
 
-    // tile shape: one consumer thread per (row, theta quad) (per pair of v
-    // rows in the two-row form), at most the largest launch-bound class (+
-    // the producer warp).  By default the rows
-    // of (y, v) with the fewest halo reads per row among the shapes whose block
-    // fits the largest class that runs without spills (640 consumer threads;
-    // 480 in fixed point), discounted by the share of the SMs the
-    // shape can keep busy (a small grid needs small tiles to fill the GPU),
-    // and as many stages as fit; hj_autotune measures the candidates instead.
+    // tile shape: one consumer thread per (row, theta quad) (per two or four v
+    // rows in the several-row forms), at most the largest launch-bound class
+    // (+ the producer warp).  By default the shape with the least step_cost()
+    // among those that fit the largest class without spills (640 consumer
+    // threads; 608 in fixed point) and leave room for 4 stages, and as many
+    // stages as fit; hj_autotune measures the candidates instead.
     const int q4 = g->p4 / 4;
     if (max_consumers(fixed) / q4 < 1) return fail("theta rows too long for one CTA");
     int ty = g->tile_req[0], tv = g->tile_req[1];
     if (ty <= 0 || tv <= 0) {
-        const int cap = fixed ? VARIANTS_Q527[1] : VARIANTS_F32[2];
+        const int cap = hj_tiled_variant(fixed, 2);
         double best = 1e300;
         int bty = 1, btv = 1;
         for (int a = 1; a <= 16 && a <= g->n[1]; ++a)
             for (int b = 1; b <= 16 && b <= g->n[2]; ++b) {
                 if ((ty > 0 && a != ty) || (tv > 0 && b != tv)) continue;
-                const int cons = consumers_of(g, a, b);
-                if (cons > cap && !(a == 1 && b == 1)) continue;
-                // room for the smallest ring (4 stages)
-                if (4 * (size_t)make_params(g, a, b, 1, 0).stage_bytes + 2048 > (size_t)maxsmem && !(a == 1 && b == 1))
-                    continue;
-                // work items this shape can offer (columns x chunks of >= 4 planes)
-                const double items = (double)((g->n[1] + a - 1) / a) * ((g->n[2] + b - 1) / b) *
-                                     (g->n[0] / 4 > 1 ? g->n[0] / 4 : 1);
-                const double busy = items < sms ? items / (sms > 0 ? sms : 1) : 1.0;
-                const double c = (double)(a + 2) * (b + 2) / (a * b) / busy - 1e-6 * a * b;  // ties: more rows
+                const TiledParams C = make_params(g, a, b, 1, 0);
+                // (fixed point: tiles of one or two rows along an axis measured slower
+                // than the estimate, 70x90x40x72 69 us at 15 x 2, 61 at 6 x 5)
+                const bool thin = fixed && ((a < 3 && g->n[1] > 2) || (b < 3 && g->n[2] > 2));
+                const bool fits = !thin && C.nconsumer <= cap && 4 * (size_t)C.stage_bytes + 2048 <= (size_t)maxsmem;
+                if (!fits && !(a == 1 && b == 1)) continue;
+                const double c = fits ? step_cost(g, C, sms > 0 ? sms : 1, g->tile_req[2]) : 1e299;
                 if (c < best) {
                     best = c;
                     bty = a;

@@ -113,6 +113,19 @@ __device__ __forceinline__ ItemGeom item_geom(const TiledParams &P, const HjGeom
     return it;
 }
 
+// The CTA's next work item.  In fixed point the order moves on by one place
+// per round: tiles at the ends of v cost more (their ghosts), and where the
+// tiles along v divide the grid size, a plain stride would give a CTA the same
+// end in every round.
+template <bool FIXED>
+__device__ __forceinline__ int next_item(int item)
+{
+    const int n = (int)gridDim.x;
+    if (!FIXED) return item + n;
+    const int place = item % n;
+    return item - place + n + (place + 1 == n ? 0 : place + 1);
+}
+
 __device__ __forceinline__ int32_t f4geti(const float4 &v, int e) { return __float_as_int(f4get(v, e)); }
 
 // FIXED: Q5.27 values (the ring and the buffers hold int32 codes).
@@ -181,7 +194,7 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
             // bytes each box delivers (the exact box sizes, not the padded room)
             const uint32_t tx_halo = (uint32_t)(P.halo_box * 4), tx_v0 = (uint32_t)(P.v0_floats * 4);
             bool ok = true;
-            for (int item = blockIdx.x; item < P.nitems && ok; item += gridDim.x) {
+            for (int item = blockIdx.x; item < P.nitems && ok; item = next_item<FIXED>(item)) {
                 ItemGeom it = item_geom(P, g, item);
                 for (int p = it.pl0; p <= it.pl1; ++p) {
                     // the slot's previous contents must have been released
@@ -309,7 +322,7 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
         if (lane == 0) mbar_arrive(&empty[rslot]);     \
         if (++rslot == nst) rslot = 0;                 \
     } while (0)
-        for (int item = blockIdx.x; item < P.nitems && ok; item += gridDim.x) {
+        for (int item = blockIdx.x; item < P.nitems && ok; item = next_item<FIXED>(item)) {
             // a producer that gave up stops the consumers at the next item (a
             // plane that never arrives ends their bounded waits instead)
             if (LEAN && __any_sync(0xffffffffu, *abort_flag != 0)) {

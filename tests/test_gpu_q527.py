@@ -215,3 +215,21 @@ def test_q527_full_size_sampled_step_parity(hj):
         st = g.solve_brt(w.T, w.cfl)
         assert st.t_final == w.T
         assert np.all(read_codes(g) <= Q0)
+
+
+@pytest.mark.parametrize("shape", [None, (1, 1, 4, 4), (2, 1, 4, 4), (1, 1, 40, 0), (4, 3, 7, 0)])
+def test_q527_items_over_several_rounds(hj, shape):
+    """CTAs that take several work items (up to 4950 of them, the order turning
+    round every other round, the last round partly filled) write every cell
+    once: the codes of the generic kernel, bit for bit."""
+    w = scenes.custom_workload((40, 45, 11, 8), 4, T=0.3)
+    V0 = scenes.initial_value(w.grid, w.scene)
+    Q, st, _ = gpu_codes(hj, w, V0, hj.HJ_KERNEL_GENERIC)
+    with hj.Grid.for_workload(w, hj.HJ_Q527) as g:
+        g.set_kernel(hj.HJ_KERNEL_TILED)
+        if shape is not None:
+            g.set_tile_shape(shape)
+        g.set_initial_value(V0)
+        st_t = g.solve_brt(w.T, w.cfl)
+        assert st_t.kernel == hj.HJ_KERNEL_TILED and st_t.steps == st.steps
+        assert np.array_equal(read_codes(g), Q)
