@@ -16,7 +16,7 @@
 // sweep is bound by shared-memory bandwidth and issue (about 31 shared-memory
 // wavefronts and 130 instructions per warp and column).  Measured, us per step
 // with the L2-resident form and with this one: 31x31x11x16 FP32 4.2 -> 2.4,
-// 60x60x20x36 FP32 12.1 -> 5.3, Q5.27 with steering 18.1 -> 10.4, 47x53x17x27
+// 60x60x20x36 FP32 12.1 -> 5.3, Q5.27 with steering 18.1 -> 8.7, 47x53x17x27
 // with steering 9.0 -> 4.0.  What was tried and is slower: V and V0 in registers
 // with the columns unrolled (spills, and 240 instructions per column: 9.5 us on
 // 60x60x20x36), the paired FP32 instructions (fewer instructions, but each
@@ -115,7 +115,8 @@ __device__ __forceinline__ bool wait_published(const unsigned int *p, unsigned i
 struct Thread {
     float K1[4], K2[4], k3, k4;  // FP32: |xdot_d| / dx_d; Q5.27: weight magnitudes (int32 bits)
     int32_t nsum[4];             // Q5.27: -(sum of the four weights)
-    bool wsmall;                 // Q5.27: none below -2^30 (hj_q527_update_interior32)
+    bool wsmall;                 // Q5.27: none below -2^30 in the warp (hj_q527_update_interior32)
+    bool edge_warp;              // Q5.27: some quad of the warp has an x or v ghost
     uint32_t mx[4], my[4];
     uint32_t sx;
     int ovm, ovp, lidx, ridx, lreal, cs;
@@ -204,14 +205,15 @@ __device__ __forceinline__ void sweep(const Thread &T, SweepIO io, const float d
             }
             if (gym) ya = yp;  // the value the ghost is formed from
             if (gyp) yb = ym;
-            const bool anyg = T.gvm || T.gvp || (T.xmix ? (T.gxm || T.gxp) : T.gu) || gym || gyp;
             const int32_t w3 = fi(T.k3), w4 = fi(T.k4);
             int32_t tt[4];  // the larger theta neighbour
             tt[0] = max(fi(PADDED && lreal == 1 ? tr : c.y), fi(tl));
             tt[1] = max(fi(PADDED && lreal == 2 ? tr : c.z), fi(c.x));
             tt[2] = max(fi(PADDED && lreal == 3 ? tr : c.w), fi(c.y));
             tt[3] = max(fi(tr), fi(c.z));
-            if (!anyg && T.wsmall) {  // every neighbour is a grid value
+            // every neighbour of the warp's quads is a grid value (a quad without ghosts gives
+            // the same codes in both forms, and a warp that splits takes the time of the two)
+            if (T.wsmall && !T.edge_warp && !gym && !gyp) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int32_t u1 = fi(MIX ? bitsel(T.mx[e], f4get(xb, e), f4get(xa, e)) : f4get(ux, e));
@@ -315,6 +317,7 @@ __global__ void __launch_bounds__(MAXT, 1)
                 T.K2[e] = fabsf(c.c2);
             }
         }
+        if (FIXED) T.wsmall = __all_sync(0xffffffffu, T.wsmall || !act);
     };
     // the sides come from the velocities; lanes whose weight is 0 (at either
     // step size) may sit on any side
@@ -374,6 +377,7 @@ __global__ void __launch_bounds__(MAXT, 1)
     T.gy0 = gy0;
     T.gy1 = gy1;
     T.gu = gu;
+    T.edge_warp = FIXED && __any_sync(0xffffffffu, act && (gvm || gvp || (T.xmix ? gxm || gxp : gu)));
     // halo columns this thread reads
     const bool need_xm = act && !xm_in && !gxm && (clx != PLUS || gxp);
     const bool need_xp = act && !xp_in && !gxp && (clx != MINUS || gxm);
