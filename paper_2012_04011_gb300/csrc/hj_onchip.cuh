@@ -16,7 +16,7 @@
 // sweep is bound by shared-memory bandwidth and issue (about 31 shared-memory
 // wavefronts and 130 instructions per warp and column).  Measured, us per step
 // with the L2-resident form and with this one: 31x31x11x16 FP32 4.2 -> 2.4,
-// 60x60x20x36 FP32 12.1 -> 5.3, Q5.27 with steering 18.1 -> 8.7, 47x53x17x27
+// 60x60x20x36 FP32 12.1 -> 5.3, Q5.27 with steering 18.1 -> 8.5, 47x53x17x27
 // with steering 9.0 -> 4.0.  What was tried and is slower: V and V0 in registers
 // with the columns unrolled (spills, and 240 instructions per column: 9.5 us on
 // 60x60x20x36), the paired FP32 instructions (fewer instructions, but each
@@ -271,12 +271,21 @@ __global__ void __launch_bounds__(MAXT, 1)
     const int N1 = g.n1, N2 = g.n2, N3 = g.n3, N4 = g.n4, P4 = g.p4, q4 = P4 / 4;
     const int cs = N3 * P4;  // values of a column: the stride along y, in shared and in global memory
     const int tid = threadIdx.x, lane = tid & 31;
-    const int q = tid % q4, rr = tid / q4, k = rr % N3;
+    const int q = tid % q4, rr = tid / q4;
     const int cx = (int)blockIdx.x / P.gy, cy = (int)blockIdx.x - cx * P.gy;
     const int x0 = cx * P.bx, y0 = cy * P.by;
     const int bxa = min(P.bx, N1 - x0), bya = min(P.by, N2 - y0);  // this block's columns
     const bool act = rr / N3 < bxa;
-    const int lx = act ? rr / N3 : 0;  // (threads past the block read the first column's, and store nothing)
+    int k = rr % N3, lx = act ? rr / N3 : 0;  // (threads past the block read the first column's, and store nothing)
+    if (FIXED && act && N3 > 2) {
+        // In fixed point a warp with an end of v takes the longer form: the ends of
+        // all the block's columns come first, so that fewer warps have one (us per
+        // step, car: 47x53x17x27 6.1 -> 5.6, 80x80x13x16 6.2 -> 5.2, 60x60x20x36
+        // 8.7 -> 8.5, 13x13x64x30 the same).
+        const int rm = rr - 2 * bxa;
+        lx = rm < 0 ? rr / 2 : rm / (N3 - 2);
+        k = rm < 0 ? (rr & 1) * (N3 - 1) : 1 + rm % (N3 - 2);
+    }
     const int x = x0 + lx;
     const int e0 = k * P4 + 4 * q;
     const int lreal = min(4, N4 - 4 * q);  // lanes of the quad inside the row
