@@ -40,7 +40,7 @@ BYTES_PER_UPDATE = {"f32": 12, "f64": 24, "q527": 12, "f32_bcast": 8}
 # kernel then reads that field instead of V0 (V_n read, V_{n+1} written: 8 B)
 F32_BYTES = BYTES_PER_UPDATE["f32_bcast"]
 KERNEL_NAMES = {1: "generic", 2: "tiled", 3: "resident"}
-PROFILE = os.path.join(ROOT, "profiles", "hj_step_tiled_car4d_128x128x64x96.md")
+PROFILE = os.path.join(ROOT, "profiles", "hj_step_tiled_bcast_car4d_128x128x64x96.md")
 KERNEL_SOURCES = ["hj_tiled_kernel.cuh", "hj_tiled_f32.cu", "hj_device.cuh", "hj_tma.cuh", "hj_internal.h"]
 # FP64 path: bound by the FP64 unit.  Algorithmic FP64 flops per cell-update
 # of the FP64 step kernel: V_new = w0 V_c + |w1| V_up1 + |w2| V_up2 + dt k3
