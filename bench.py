@@ -761,7 +761,7 @@ def run_ours(args):
             "value": r64["value"], "unit": UNIT, "ms_per_step": r64["ms_per_step"], "steps": r64["K"],
             "latency_ms": r64["latency_ms"], "avg_step_kernel_ms": r64["avg_step_kernel_ms"],
             "hbm_frac": BYTES_PER_UPDATE["f64"] * ncell / (r64["avg_step_kernel_ms"] * 1e-3) / 1e9 / peak,
-            "roofline": {"bound": "alu", "kernel": "hj_step_generic_kernel<double>", "achieved": a64,
+            "roofline": {"bound": "alu", "kernel": "hj_step_fp64_kernel", "achieved": a64,
                          "peak": fpk, "unit": "TFLOP/s", "frac": a64 / fpk, "peak_source": fpk_src,
                          "flops_per_update": FP64_FLOPS_PER_UPDATE,
                          "flops_counted": "1 DMUL + 4 DFMA per cell-update (dt folded into the coefficient table)"},
