@@ -141,18 +141,21 @@ double heaviest_q527(const hj_grid *g, const TiledParams &P, int xc, int nchunk,
 // plane).  A plane costs a fixed part (the waits on its stage and the release)
 // and a part per consumer warp that depends on the launch-bound class, which
 // sets the registers; the forms that read V0 as a field also pay for the bytes
-// through shared memory.  Below 8 warps an SM is latency-bound and a plane
-// takes as long as with 8.  In fixed point the tiles' costs differ and the CTA
-// with the heaviest items sets the time.  Coefficients: least squares over the
-// 20 to 40 shapes that hj_autotune timed on each of 10 grids (2 to 101 M
-// cells; in fixed point 18, of which 4 were not in the fit).  Against the best
-// timed shape of each grid the picks take 1.00 to 1.03 times as long with a 4D
-// V0, 1.00 to 1.26 (mean 1.04) with the field and 1.00 to 1.11 (1.02) in fixed
-// point; the shape with the fewest halo reads per row, the rule before, took
-// 1.00 to 1.33 (1.13), 1.03 to 1.26 (1.16) and 1.00 to 1.74 (1.22).  Per step:
-// 80x80x25x40 FP32 18.4 -> 15.4 us, 128x128x64x96 with the field 156 -> 141,
-// 64x64x24x36 Q5.27 35.0 -> 16.0, 100x100x30x48 Q5.27 69.5 -> 55.2,
-// 113x97x47x59 Q5.27 156 -> 109.
+// through shared memory.  Below 8 warps (11 with several rows a thread) an SM
+// is latency-bound and a plane takes as long as with that many.  In fixed
+// point the tiles' costs differ and the CTA with the heaviest items sets the
+// time.  Coefficients: least squares over the 20 to 40 shapes that
+// hj_autotune timed on each of 10 grids (2 to 101 M cells; 18 in fixed point).
+// Against the best timed shape of each grid the picks take 1.00 to 1.03 times
+// as long with a 4D V0 (mean 1.01), 1.00 to 1.11 (1.02; 6 of the 16 grids not
+// in the fit) with the field and 1.00 to 1.18 (1.04) in fixed point (fitted
+// when a warp with and without ghosts ran both forms, 1.00 to 1.11 then; a fit
+// to the present kernel with the 736 class gained up to 15 % on 7 of the 18
+// grids and lost up to 14 % on 4); the shape with the fewest halo reads per
+// row, the rule before, took 1.00 to 1.33 (1.13), 1.03 to 1.26 (1.16) and 1.00
+// to 1.74 (1.22).  Per step, that rule and this one: 80x80x25x40 FP32 18.4 and
+// 15.4 us, 128x128x64x96 with the field 156 and 141, 128x128x30x16 with the
+// field 20.3 and 17.9.
 double step_cost(const hj_grid *g, const TiledParams &P, int slots, int xc_req)
 {
     static const double F4D[4] = {0.0089, 0.0111, 0.0148, 0.0210}, FXY[4] = {0.0169, 0.0147, 0.0176, 0.0209},
@@ -162,7 +165,7 @@ double step_cost(const hj_grid *g, const TiledParams &P, int slots, int xc_req)
     const int nchunk = (g->n[0] + xc - 1) / xc;
     int cls = 0;
     while (cls < 3 && P.nconsumer > hj_tiled_variant(fixed, cls)) ++cls;
-    const double warps = P.nconsumer > 256 ? P.nconsumer / 32 : 8;
+    const double least = P.rpt > 1 ? 11 : 8, warps = P.nconsumer / 32 > least ? P.nconsumer / 32 : least;
     const long long rounds = ((long long)P.ncol * nchunk + slots - 1) / slots;
     const double planes = (double)rounds * (xc + (nchunk > 1 ? 2 : 1));
     if (fixed) return heaviest_q527(g, P, xc, nchunk, slots) * warps * Q[cls] + planes * 0.25;
