@@ -328,15 +328,16 @@ __global__ void __launch_bounds__(MAXT, 1)
         }
         if (FIXED) T.wsmall = __all_sync(0xffffffffu, T.wsmall || !act);
     };
-    // the sides come from the velocities; lanes whose weight is 0 (at either
-    // step size) may sit on any side
+    // the sides come from the velocities; lanes whose weight is 0 (at each step
+    // size this launch takes: the cut step's table is built only for a call
+    // that has one) may sit on any side
     {
         uint32_t wx = 0u, wy = 0u;
         for (int e = 0; e < lreal; ++e) {
             const uint32_t bit = 1u << e;
             if constexpr (FIXED) {
                 const HjCoef<double> c = ((const HjCoef<double> *)coefp)[k * N4 + 4 * q + e];
-                const int32_t *w1 = qw + hj_qw_count(N3, P4);
+                const int32_t *w1 = P.cut ? qw + hj_qw_count(N3, P4) : qw;
                 if (c.c1 >= 0.0) sx |= bit;
                 if (c.c2 >= 0.0) sy |= bit;
                 if (qw[e0 + e] | w1[e0 + e]) wx |= bit;

@@ -63,3 +63,32 @@ def test_onchip_equals_generic(hj, n, prec, flat):
         for chunk in (None, 2, 3):
             got, s2 = solve(hj, n, code, hj.HJ_KERNEL_RESIDENT, V0, steer, chunk, lo)
             assert s2 == steps and np.array_equal(got, ref), (steer, chunk)
+
+
+@pytest.mark.parametrize("n4", [16, 32, 48])
+@pytest.mark.parametrize("steer", [False, True])
+def test_onchip_q527_ignores_weights_of_earlier_dynamics(hj, n4, steer):
+    """A call that does not reach its horizon has no cut step and builds no
+    table for one: whatever the second weight table holds (here the weights of
+    the constant dynamics solved before, nonzero in every lane) takes no part.
+    With N4 a multiple of 16 the quad that starts at theta = pi/2 has a lane of
+    weight 0 whose cosine (6e-17) differs in sign from the other three's."""
+    n = (31, 31, 11, n4)
+    w = scenes.custom_workload(n, n_circles=4, seed=3)
+    V0 = scenes.initial_value(w.grid, w.scene)
+    out = []
+    for kernel in (hj.HJ_KERNEL_GENERIC, hj.HJ_KERNEL_RESIDENT):
+        with hj.Grid(n, scenes.DOMAIN_LO, scenes.DOMAIN_HI, scenes.PERIODIC_THETA, hj.HJ_Q527) as g:
+            g.set_kernel(kernel)
+            g.set_dynamics(hj.HJ_DYN_CONST, (1.0, 1.0, 0.0, 0.0))
+            g.set_initial_value(V0)
+            g.solve_brt(0.4, scenes.CFL)
+            if steer:
+                g.set_dynamics(hj.HJ_DYN_CAR4D_STEER, STEER)
+            else:
+                g.set_dynamics(hj.HJ_DYN_CAR4D, (scenes.A_MAX, scenes.W_MAX))
+            g.set_initial_value(V0)
+            st = g.advance_brt(0.4, scenes.CFL, 3)
+            assert st.kernel == kernel and st.steps == 3
+            out.append(g.read_value())
+    assert np.array_equal(out[0], out[1])
