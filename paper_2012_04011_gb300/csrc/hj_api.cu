@@ -207,6 +207,18 @@ hj_status wait_stream(const hj_grid *g)
     return HJ_OK;
 }
 
+// Refuses a stream that the caller is capturing, before anything is changed:
+// work queued there does not run, and t, the step count and the step sizes the
+// device holds are kept on the host, which would take it as done.
+hj_status refuse_capture(const hj_grid *g)
+{
+    cudaStreamCaptureStatus cs;
+    HJ_CUDA(cudaStreamIsCapturing(g->stream, &cs));
+    if (cs != cudaStreamCaptureStatusNone)
+        return set_err(HJ_ERR_CUDA, "the grid's stream is being captured (this call waits for its own work)");
+    return HJ_OK;
+}
+
 // The flags, as the host reads them after a synchronisation.
 int read_status(const hj_grid *g) { return *(volatile int *)&g->hflags->status; }
 
@@ -834,6 +846,7 @@ hj_status hj_set_initial_value(hj_grid *g, const double *v0, size_t count)
     if (count != (size_t)g->ncell)
         return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2*N3*N4 = %lld", count, g->ncell);
     if ((s = activate(g)) != HJ_OK) return s;
+    if ((s = refuse_capture(g)) != HJ_OK) return s;
     reset_state(g);
     // pinned host memory: the ingest kernel reads it directly; otherwise stage
     // the dense FP64 array in the ping-pong region (2 * nint * esize >= ncell * 8 bytes)
@@ -854,6 +867,7 @@ hj_status hj_set_initial_value_xy(hj_grid *g, const double *v0_xy, size_t count)
     const long long nxy = (long long)g->n[0] * g->n[1];
     if (count != (size_t)nxy) return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2 = %lld", count, nxy);
     if ((s = activate(g)) != HJ_OK) return s;
+    if ((s = refuse_capture(g)) != HJ_OK) return s;
     reset_state(g);
     double *staging = (double *)g->buf;  // N1*N2 doubles fit in the ping-pong region
     HJ_CUDA(cudaMemcpyAsync(staging, v0_xy, sizeof(double) * (size_t)nxy, cudaMemcpyHostToDevice, g->stream));
@@ -870,6 +884,7 @@ hj_status hj_set_initial_value_xy_device(hj_grid *g, const void *v0_xy_device, h
     const long long nxy = (long long)g->n[0] * g->n[1];
     if (count != (size_t)nxy) return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2 = %lld", count, nxy);
     if ((s = activate(g)) != HJ_OK) return s;
+    if ((s = refuse_capture(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;
     reset_state(g);
     return ingest_xy(g, v0_xy_device, dtype, nxy);
@@ -885,6 +900,7 @@ hj_status hj_set_initial_value_device(hj_grid *g, const void *v0_device, hj_prec
     if (count != (size_t)g->ncell)
         return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2*N3*N4 = %lld", count, g->ncell);
     if ((s = activate(g)) != HJ_OK) return s;
+    if ((s = refuse_capture(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;
     reset_state(g);
     return ingest_4d(g, v0_device, dtype);
@@ -915,6 +931,7 @@ static hj_status advance_loop(hj_grid *g, double T, double cfl, int64_t max_step
     if (!g->has_dyn) return set_err(HJ_ERR_STATE, "hj_set_dynamics has not been called");
     if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
     if ((s = activate(g)) != HJ_OK) return s;
+    if ((s = refuse_capture(g)) != HJ_OK) return s;
 
     const hj_kernel kern = effective_kernel(g);
     int launches = 0;
@@ -1230,6 +1247,7 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
     if (!g->tiled_ok) return set_err(HJ_ERR_UNSUPPORTED, "this grid has no tiled kernel");
     if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
     if ((s = activate(g)) != HJ_OK) return s;
+    if ((s = refuse_capture(g)) != HJ_OK) return s;
     if (g->nstep != 0) return set_err(HJ_ERR_STATE, "autotune must run before the first step");
     double dt_trial = 0.0;
     if (!cfl_step(g, 0.8, &dt_trial)) return set_err(HJ_ERR_UNSTABLE, "the CFL step is not a usable number");
