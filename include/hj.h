@@ -528,6 +528,13 @@ HJ_API hj_status hj_wait_selftest(int64_t limit_ns, int32_t *status, int64_t *wa
  * side effects as hj_wait_selftest. */
 HJ_API hj_status hj_barrier_selftest(int64_t limit_ns, int32_t *status, int64_t *waited_ns);
 
+/* Test of a step launch that fails: of the step launches that follow on g
+ * (one per step; one per call of HJ_KERNEL_RESIDENT), number `launch` (1, 2,
+ * ...; 0: none) fails on the host without being made.  The call that meets it
+ * returns HJ_ERR_CUDA; the steps queued before it have run and count, so the
+ * value, t and the step count stay those of one another. */
+HJ_API hj_status hj_launch_selftest(hj_grid *g, int64_t launch);
+
 /* FP64 fused multiply-add throughput probe.  The paper has no counterpart:
  * it measures the FP64 rate that the FP64 step kernel and the query kernel
  * are held against (their roofline).  Launches one kernel on cuda_stream

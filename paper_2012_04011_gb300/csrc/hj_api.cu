@@ -222,6 +222,13 @@ hj_status refuse_capture(const hj_grid *g)
 // The flags, as the host reads them after a synchronisation.
 int read_status(const hj_grid *g) { return *(volatile int *)&g->hflags->status; }
 
+hj_status need_value(const hj_grid *g)
+{
+    if (g->has_value) return HJ_OK;
+    return set_err(HJ_ERR_STATE, g->value_lost ? "the value was lost in a call that failed; set an initial value"
+                                               : "no initial value (hj_set_initial_value)");
+}
+
 hj_status upload_tables(hj_grid *g)
 {
     const int N3 = g->n[2], N4 = g->n[3], P4 = g->p4;
@@ -361,15 +368,27 @@ hj_kernel effective_kernel(const hj_grid *g)
     return g->tiled_ok ? HJ_KERNEL_TILED : HJ_KERNEL_GENERIC;
 }
 
+// Whether this launch is the one hj_launch_selftest makes fail.
+bool fail_selftest(hj_grid *g) { return g->fail_in > 0 && --g->fail_in == 0; }
+
+hj_status launched(cudaError_t e)
+{
+    if (e == cudaSuccess) return HJ_OK;
+    cudaGetLastError();  // a failed call (not a sticky fault) must not fail later checks
+    return set_err(e == cudaErrorMemoryAllocation ? HJ_ERR_OOM : HJ_ERR_CUDA, "step launch: %s",
+                   cudaGetErrorString(e));
+}
+
 hj_status launch_step(hj_grid *g, hj_kernel k, long long n, int sel)
 {
-    cudaError_t e = (k == HJ_KERNEL_TILED) ? hj_launch_step_tiled(g, n, sel) : hj_launch_step_generic(g, n, sel);
-    if (e != cudaSuccess) {
-        cudaGetLastError();  // a failed call (not a sticky fault) must not fail later checks
-        return set_err(e == cudaErrorMemoryAllocation ? HJ_ERR_OOM : HJ_ERR_CUDA, "step launch: %s",
-                       cudaGetErrorString(e));
-    }
-    return HJ_OK;
+    return launched(fail_selftest(g)           ? cudaErrorLaunchOutOfResources
+                    : (k == HJ_KERNEL_TILED) ? hj_launch_step_tiled(g, n, sel)
+                                             : hj_launch_step_generic(g, n, sel));
+}
+
+hj_status launch_resident(hj_grid *g, long long n, long long k, bool cut)
+{
+    return launched(fail_selftest(g) ? cudaErrorLaunchOutOfResources : hj_launch_step_resident(g, n, k, cut));
 }
 
 // Grids below this many cells take a step in a few microseconds, less than
@@ -383,7 +402,7 @@ constexpr long long GRAPH_MAX_CELLS = 1LL << 24;
 bool launch_steps_graph(hj_grid *g, hj_kernel kern, long long n, long long k, bool cut)
 {
     const int parity = n == 0 ? 0 : 1 + (int)((n - 1) & 1);
-    if (g->ncell >= GRAPH_MAX_CELLS || k < 4 || k > 4096) return false;
+    if (g->ncell >= GRAPH_MAX_CELLS || k < 4 || k > 4096 || g->fail_in > 0) return false;
     cudaStreamCaptureStatus cs;
     if (cudaStreamIsCapturing(g->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
     int hit = -1, victim = 0;
@@ -807,6 +826,7 @@ static hj_status finish_ingest(hj_grid *g)
         return set_err(HJ_ERR_INVALID_ARG, "V0 contains NaN or Inf");
     }
     g->has_value = true;
+    g->value_lost = false;
     return HJ_OK;
 }
 
@@ -916,8 +936,20 @@ static hj_status advance_impl(hj_grid *g, double T, double cfl, int64_t max_step
 {
     // the step kernels that also reduce the change run only in this call
     g->track = threshold > 0.0;
+    g->uncounted = false;
     const hj_status s = advance_loop(g, T, cfl, max_steps, threshold, stats);
     g->track = false;
+    if (s != HJ_OK) {
+        // the device may not hold the step sizes; steps that ran and were not counted
+        // (a wait that timed out, a failed synchronisation) leave no known value
+        g->up_dt[0] = g->up_dt[1] = -1.0;
+        if (g->uncounted) {
+            cudaStreamSynchronize(g->stream);
+            cudaGetLastError();
+            g->has_value = false;
+            g->value_lost = true;
+        }
+    }
     return s;
 }
 
@@ -929,16 +961,19 @@ static hj_status advance_loop(hj_grid *g, double T, double cfl, int64_t max_step
     if (!isfinite(cfl) || !(cfl > 0) || cfl > 1) return set_err(HJ_ERR_INVALID_ARG, "cfl must be in (0, 1]");
     if (max_steps < 0) return set_err(HJ_ERR_INVALID_ARG, "max_steps must be >= 0");
     if (!g->has_dyn) return set_err(HJ_ERR_STATE, "hj_set_dynamics has not been called");
-    if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
+    if (read_status(g) != HJ_OK)
+        return set_err((hj_status)read_status(g), "device reported %s", hj_status_string((hj_status)read_status(g)));
+    if ((s = need_value(g)) != HJ_OK) return s;
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = refuse_capture(g)) != HJ_OK) return s;
 
     const hj_kernel kern = effective_kernel(g);
     int launches = 0;
     double dt = 0.0;
-    if (read_status(g) == HJ_OK && g->t < T && !cfl_step(g, cfl, &dt)) g->hflags->status = HJ_ERR_UNSTABLE;
-    if (read_status(g) != HJ_OK)
-        return set_err((hj_status)read_status(g), "device reported %s", hj_status_string((hj_status)read_status(g)));
+    if (g->t < T && !cfl_step(g, cfl, &dt)) {
+        g->hflags->status = HJ_ERR_UNSTABLE;
+        return set_err(HJ_ERR_UNSTABLE, "device reported %s", hj_status_string(HJ_ERR_UNSTABLE));
+    }
     HJ_CUDA(cudaEventRecord(g->ev[0], g->stream));
     const long long n_start = g->nstep;
     double t = g->t, dt_first = 0.0, dt_last = 0.0, last_change = 0.0;
@@ -963,19 +998,24 @@ static hj_status advance_loop(hj_grid *g, double T, double cfl, int64_t max_step
             HJ_CUDA(cudaEventRecord(g->ev[1], g->stream));
             loop_started = true;
         }
+        // (after a launch that fails, the steps queued before it still run: they
+        // are waited for and counted before the call returns the error)
+        long long taken = 0;
+        g->uncounted = true;
         if (kern == HJ_KERNEL_RESIDENT) {
-            HJ_CUDA(hj_launch_step_resident(g, g->nstep, k, cut));
-            ++launches;
-        } else if (launch_steps_graph(g, kern, g->nstep, k, cut)) {
-            launches += (int)k;
-        } else {
-            for (long long i = 0; i < k; ++i) {
-                if ((s = launch_step(g, kern, g->nstep + i, cut && i == k - 1)) != HJ_OK) return s;
+            if ((s = launch_resident(g, g->nstep, k, cut)) == HJ_OK) {
+                taken = k;
                 ++launches;
             }
+        } else if (launch_steps_graph(g, kern, g->nstep, k, cut)) {
+            taken = k;
+            launches += (int)k;
+        } else {
+            while (taken < k && (s = launch_step(g, kern, g->nstep + taken, cut && taken == k - 1)) == HJ_OK) ++taken;
+            launches += (int)taken;
         }
+        const hj_status queued = s;
         HJ_CUDA(cudaEventRecord(g->ev[2], g->stream));
-        long long taken = k;
         if (threshold > 0.0) {
             HJ_CUDA(cudaMemcpyAsync(g->hloop, g->loop, sizeof(HjLoop), cudaMemcpyDeviceToHost, g->stream));
             HJ_CUDA(cudaEventRecord(g->ev[3], g->stream));
@@ -998,6 +1038,8 @@ static hj_status advance_loop(hj_grid *g, double T, double cfl, int64_t max_step
         }
         g->t = t;
         g->nstep += taken;
+        g->uncounted = false;
+        if (queued != HJ_OK) return queued;
     }
     if (!loop_started) {
         HJ_CUDA(cudaEventRecord(g->ev[3], g->stream));
@@ -1058,7 +1100,7 @@ hj_status hj_read_value(const hj_grid *gc, double *out, size_t count)
     if (!out) return set_err(HJ_ERR_INVALID_ARG, "out is NULL");
     if (count != (size_t)g->ncell)
         return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2*N3*N4 = %lld", count, g->ncell);
-    if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
+    if ((s = need_value(g)) != HJ_OK) return s;
     if ((s = activate(g)) != HJ_OK) return s;
     const long long n = g->nstep;
     const void *src = hj_value_ptr(g, n);
@@ -1116,7 +1158,7 @@ hj_status hj_query_device(const hj_grid *gc, const double *states, int64_t m, do
     if (s != HJ_OK) return s;
     if (m < 0) return set_err(HJ_ERR_INVALID_ARG, "m must be >= 0");
     if (m > 0 && (!states || !value)) return set_err(HJ_ERR_INVALID_ARG, "states and value must not be NULL");
-    if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
+    if ((s = need_value(g)) != HJ_OK) return s;
     if (control && !g->has_dyn) return set_err(HJ_ERR_STATE, "the control needs the dynamics (hj_set_dynamics)");
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;
@@ -1133,7 +1175,7 @@ hj_status hj_query(const hj_grid *gc, const double *states, int64_t m, double *v
     if (s != HJ_OK) return s;
     if (m < 0) return set_err(HJ_ERR_INVALID_ARG, "m must be >= 0");
     if (m > 0 && (!states || !value)) return set_err(HJ_ERR_INVALID_ARG, "states and value must not be NULL");
-    if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
+    if ((s = need_value(g)) != HJ_OK) return s;
     if (control && !g->has_dyn) return set_err(HJ_ERR_STATE, "the control needs the dynamics (hj_set_dynamics)");
     if ((s = activate(g)) != HJ_OK) return s;
     const long long n = g->nstep;
@@ -1177,7 +1219,7 @@ hj_status hj_read_value_device(const hj_grid *gc, void *out_device, hj_precision
     if (!valid_prec(dtype)) return set_err(HJ_ERR_INVALID_ARG, "unknown dtype");
     if (count != (size_t)g->ncell)
         return set_err(HJ_ERR_INVALID_ARG, "count %zu != N1*N2*N3*N4 = %lld", count, g->ncell);
-    if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
+    if ((s = need_value(g)) != HJ_OK) return s;
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = follow_default_stream(g)) != HJ_OK) return s;  // the output array too
     const void *src = hj_value_ptr(g, g->nstep);
@@ -1245,12 +1287,13 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
     if (steps_per_trial < 1) return set_err(HJ_ERR_INVALID_ARG, "steps_per_trial must be >= 1");
     if (max_results < 0) return set_err(HJ_ERR_INVALID_ARG, "max_results must be >= 0");
     if (!g->tiled_ok) return set_err(HJ_ERR_UNSUPPORTED, "this grid has no tiled kernel");
-    if (!g->has_value) return set_err(HJ_ERR_STATE, "no initial value (hj_set_initial_value)");
+    if ((s = need_value(g)) != HJ_OK) return s;
     if ((s = activate(g)) != HJ_OK) return s;
     if ((s = refuse_capture(g)) != HJ_OK) return s;
     if (g->nstep != 0) return set_err(HJ_ERR_STATE, "autotune must run before the first step");
     double dt_trial = 0.0;
     if (!cfl_step(g, 0.8, &dt_trial)) return set_err(HJ_ERR_UNSTABLE, "the CFL step is not a usable number");
+    const int status0 = read_status(g);
     int32_t keep[4];
     memcpy(keep, g->tile_req, sizeof(keep));
 
@@ -1378,6 +1421,12 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
             }
         }
     }
+    if (s != HJ_OK) {  // V0, t and the step count are as before the trials; so is the status
+        cudaStreamSynchronize(g->stream);
+        cudaGetLastError();
+        g->up_dt[0] = g->up_dt[1] = -1.0;
+        g->hflags->status = status0;
+    }
     // keep the winner (or the previous shape if nothing ran)
     if (best < 1e300)
         memcpy(g->tile_req, best_req, sizeof(best_req));
@@ -1393,6 +1442,16 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
                     best_req[1], best_req[2], best_req[3], g->tile_ty, g->tile_tv, g->tile_xc, g->tile_stages);
     if (nresults) *nresults = count;
     return s;
+}
+
+hj_status hj_launch_selftest(hj_grid *g, int64_t launch)
+{
+    g_err[0] = 0;
+    hj_status s = check_grid(g);
+    if (s != HJ_OK) return s;
+    if (launch < 0) return set_err(HJ_ERR_INVALID_ARG, "launch must be >= 0");
+    g->fail_in = launch;
+    return HJ_OK;
 }
 
 hj_status hj_get_info(const hj_grid *g, hj_grid_info *info)

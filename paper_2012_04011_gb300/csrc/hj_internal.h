@@ -142,6 +142,9 @@ struct hj_grid {
     double up_dt[2];       // step sizes the device constants and dt-scaled tables hold (0: none)
 
     bool has_dyn, has_value;
+    bool value_lost;       // no value because a call failed after steps had run that it could not count
+    bool uncounted;        // the running solve call has queued steps that t and nstep do not hold yet
+    long long fail_in;     // hj_launch_selftest: the step launch from here that fails (0: none)
     hj_dynamics dyn;
     double params[4];
     HjGeom geom;

@@ -162,6 +162,7 @@ _SIGS = {
                                         ctypes.POINTER(ctypes.c_int64)]),
     "hj_barrier_selftest": (ctypes.c_int, [ctypes.c_int64, ctypes.POINTER(ctypes.c_int32),
                                            ctypes.POINTER(ctypes.c_int64)]),
+    "hj_launch_selftest": (ctypes.c_int, [_VP, ctypes.c_int64]),
     "hj_fp64_fma_probe": (ctypes.c_int, [ctypes.c_int64, ctypes.c_int32, _VP, ctypes.POINTER(ctypes.c_int64)]),
     "hj_read_value": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_double), ctypes.c_size_t]),
     "hj_read_value_device": (ctypes.c_int, [_VP, _VP, ctypes.c_int, ctypes.c_size_t]),
@@ -372,6 +373,11 @@ def hj_barrier_selftest(limit_ns: int):
     waited = ctypes.c_int64(0)
     _check(lib.hj_barrier_selftest(int(limit_ns), ctypes.byref(st), ctypes.byref(waited)))
     return int(st.value), int(waited.value)
+
+
+def hj_launch_selftest(g, launch: int):
+    """Makes step launch number `launch` (1, 2, ...; 0: none) from here fail on the host."""
+    _check(lib.hj_launch_selftest(g, int(launch)))
 
 
 def hj_read_value(g, out: np.ndarray | None = None, shape=None) -> np.ndarray:

@@ -1,5 +1,6 @@
 """Calls that fail leave a grid as it was, or say that its value is gone: a
-call on a stream that is being captured."""
+call on a stream that is being captured, a step launch that fails (on the
+host: no kernel of it runs)."""
 import numpy as np
 import pytest
 
@@ -64,3 +65,62 @@ def test_call_on_a_captured_stream_changes_nothing(hj, prec, kernel):
             assert np.array_equal(g.read_value(), v5)
         g.solve_brt(w.T, w.cfl)
         assert np.array_equal(g.read_value(), ref)
+
+
+def raw(hj, g, torch):
+    out = torch.empty(tuple(g.info().n), device="cuda",
+                      dtype={hj.HJ_FP64: torch.float64, hj.HJ_FP32: torch.float32, hj.HJ_Q527: torch.int32}[g.info().precision])
+    return g.read_value_device(out).cpu().numpy()
+
+
+@pytest.mark.parametrize("prec, kernel", [("FP64", "GENERIC"), ("FP32", "GENERIC"), ("FP32", "TILED"),
+                                          ("Q527", "TILED"), ("Q527", "GENERIC"), ("FP32", "RESIDENT"),
+                                          ("FP64", "RESIDENT"), ("Q527", "RESIDENT")])
+@pytest.mark.parametrize("first", [0, 3])
+def test_failed_launch_keeps_value_and_step_count_together(hj, prec, kernel, first):
+    """The launch of step `first` + 6 fails: six steps less one were queued
+    before it (none with the resident kernel, whose launch is a whole call)."""
+    import torch
+    w = scenes.workload("car4d_31x31x11x16")
+    V0 = scenes.initial_value(w.grid, w.scene)
+    ran = 0 if kernel == "RESIDENT" else 5
+    with hj.Grid.for_workload(w, getattr(hj, "HJ_" + prec)) as g:
+        g.set_kernel(getattr(hj, "HJ_KERNEL_" + kernel))
+        g.set_initial_value(V0)
+        st = g.advance_brt(w.T, w.cfl, first + ran)
+        after, t_after = raw(hj, g, torch), st.t_final
+        g.solve_brt(w.T, w.cfl)
+        end = raw(hj, g, torch)
+        for call in (lambda: g.solve_brt(w.T, w.cfl), lambda: g.solve_converged(1e-9, w.T, w.cfl)):
+            g.set_initial_value(V0)
+            if first:
+                g.advance_brt(w.T, w.cfl, first)
+            hj.hj_launch_selftest(g.handle, ran + 1)
+            with pytest.raises(hj.HjError) as e:
+                call()
+            assert e.value.status == hj.HJ_ERR_CUDA
+            info = g.info()
+            assert info.has_value and info.total_steps == first + ran and info.t == t_after
+            assert np.array_equal(raw(hj, g, torch), after)
+            st = g.solve_brt(w.T, w.cfl)
+            assert np.array_equal(raw(hj, g, torch), end)
+
+
+def test_failed_autotune_leaves_the_grid_ready(hj):
+    w = scenes.workload("car4d_31x31x11x16")
+    V0 = scenes.initial_value(w.grid, w.scene)
+    with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+        g.set_kernel(hj.HJ_KERNEL_TILED)
+        g.set_initial_value(V0)
+        tile = list(g.info().tile)
+        hj.hj_launch_selftest(g.handle, 3)
+        with pytest.raises(hj.HjError):
+            g.autotune(4)
+        assert list(g.info().tile) == tile and g.info().total_steps == 0
+        g.solve_brt(w.T, w.cfl)
+        V = g.read_value()
+    with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+        g.set_kernel(hj.HJ_KERNEL_TILED)
+        g.set_initial_value(V0)
+        g.solve_brt(w.T, w.cfl)
+        assert np.array_equal(g.read_value(), V)
