@@ -535,6 +535,14 @@ HJ_API hj_status hj_barrier_selftest(int64_t limit_ns, int32_t *status, int64_t 
  * value, t and the step count stay those of one another. */
 HJ_API hj_status hj_launch_selftest(hj_grid *g, int64_t launch);
 
+/* Test of the steps queued behind one whose wait ran out, without the wait:
+ * solves g (which must use HJ_KERNEL_TILED, with a V0 and no step taken) to T
+ * (threshold as hj_solve_converged; 0: none) with the flags of a timed-out
+ * step set on the device before the first one.  Returns HJ_ERR_TIMEOUT as such
+ * a solve does; *stored = 0 if every step left without storing a value.  The
+ * value is lost then, as after a timeout. */
+HJ_API hj_status hj_stop_selftest(hj_grid *g, double T, double cfl, double threshold, int32_t *stored);
+
 /* FP64 fused multiply-add throughput probe.  The paper has no counterpart:
  * it measures the FP64 rate that the FP64 step kernel and the query kernel
  * are held against (their roofline).  Launches one kernel on cuda_stream

@@ -151,6 +151,7 @@ __global__ void prologue_kernel(HjLoop *lp, const PrologueArgs a, const HjGeom g
         lp->delta_bits = 0ull;
         lp->taken = 0;
         lp->done = 0;
+        lp->stop = 0;
         lp->blocks_done = 0u;
     }
     for (int i = 0; i < 2; ++i) {
@@ -161,6 +162,13 @@ __global__ void prologue_kernel(HjLoop *lp, const PrologueArgs a, const HjGeom g
             hj_rescale_qweights(qw + i * hj_qw_count(g.n3, g.p4), coef, g.n3, g.n4, g.p4, g.k3, k4, a.dt[i], first,
                                 stride);
     }
+}
+
+// What a step whose wait ran out leaves behind (hj_stop_selftest).
+__global__ void mark_stop_kernel(HjLoop *lp, HjFlags *flags)
+{
+    *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
+    lp->stop = 1;
 }
 
 // Start of a batch slot's solve (the slot's time loop runs on the device).
@@ -994,6 +1002,7 @@ static hj_status advance_loop(hj_grid *g, double T, double cfl, int64_t max_step
             ++k;
         }
         if ((s = launch_prologue(g, dt, dt_cut, threshold, &launches)) != HJ_OK) return s;
+        if (g->stop_selftest) mark_stop_kernel<<<1, 1, 0, g->stream>>>(g->loop, g->dflags);
         if (!loop_started) {
             HJ_CUDA(cudaEventRecord(g->ev[1], g->stream));
             loop_started = true;
@@ -1452,6 +1461,34 @@ hj_status hj_launch_selftest(hj_grid *g, int64_t launch)
     if (launch < 0) return set_err(HJ_ERR_INVALID_ARG, "launch must be >= 0");
     g->fail_in = launch;
     return HJ_OK;
+}
+
+hj_status hj_stop_selftest(hj_grid *g, double T, double cfl, double threshold, int32_t *stored)
+{
+    g_err[0] = 0;
+    hj_status s = check_grid(g);
+    if (s != HJ_OK) return s;
+    if (!stored) return set_err(HJ_ERR_INVALID_ARG, "stored is NULL");
+    if (effective_kernel(g) != HJ_KERNEL_TILED) return set_err(HJ_ERR_UNSUPPORTED, "only the tiled kernel's steps wait");
+    if (!(threshold >= 0) || !isfinite(threshold)) return set_err(HJ_ERR_INVALID_ARG, "threshold must be finite and >= 0");
+    if ((s = need_value(g)) != HJ_OK) return s;
+    if (g->nstep != 0) return set_err(HJ_ERR_STATE, "the self-test must run before the first step");
+    if ((s = activate(g)) != HJ_OK) return s;
+    if ((s = refuse_capture(g)) != HJ_OK) return s;
+    const size_t bytes = 2 * (size_t)g->nint * g->esize;
+    HJ_CUDA(cudaMemsetAsync(g->buf, 0xFF, bytes, g->stream));
+    g->stop_selftest = true;
+    s = advance_impl(g, T, cfl, INT64_MAX, threshold, nullptr);
+    g->stop_selftest = false;
+    unsigned char *h = (unsigned char *)malloc(bytes);
+    if (!h) return set_err(HJ_ERR_OOM, "host allocation failed");
+    const cudaError_t e = cudaMemcpy(h, g->buf, bytes, cudaMemcpyDeviceToHost);
+    *stored = 0;
+    for (size_t i = 0; i < bytes; ++i)
+        if (h[i] != 0xFF) *stored = 1;
+    free(h);
+    HJ_CUDA(e);
+    return s;
 }
 
 hj_status hj_get_info(const hj_grid *g, hj_grid_info *info)

@@ -47,6 +47,7 @@ struct HjLoop {
     unsigned long long delta_bits;  // its running maximum (FP64 bit pattern)
     long long taken;                // steps taken since the prologue
     int done;                       // converged: later steps exit at once
+    int stop;                       // a wait of an earlier step timed out: later steps exit at once
     unsigned int blocks_done;       // CTAs of the current step that have finished
 };
 
@@ -144,6 +145,7 @@ struct hj_grid {
     bool has_dyn, has_value;
     bool value_lost;       // no value because a call failed after steps had run that it could not count
     bool uncounted;        // the running solve call has queued steps that t and nstep do not hold yet
+    bool stop_selftest;    // hj_stop_selftest: the next steps queued find an earlier one timed out
     long long fail_in;     // hj_launch_selftest: the step launch from here that fails (0: none)
     hj_dynamics dyn;
     double params[4];

@@ -46,7 +46,8 @@
 // variant.  Each cell's arithmetic is the one-row form's, in the same order.
 // Every mbarrier wait is bounded by %globaltimer; on timeout the kernel
 // records HJ_ERR_TIMEOUT in the grid's flags, stops issuing work, waits
-// (bounded) for its own copies in flight and returns.
+// (bounded) for its own copies in flight and returns; the steps queued behind
+// it see HjLoop::stop and leave at once.
 #pragma once
 
 #include <math.h>
@@ -126,6 +127,14 @@ __device__ __forceinline__ int next_item(int item)
     return item - place + n + (place + 1 == n ? 0 : place + 1);
 }
 
+// A wait ran out: the host reads the flag after the call, the steps queued
+// behind this one read the device's.
+__device__ __forceinline__ void step_timed_out(HjFlags *flags, HjLoop *loop)
+{
+    *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
+    *(volatile int *)&loop->stop = 1;
+}
+
 __device__ __forceinline__ int32_t f4geti(const float4 &v, int e) { return __float_as_int(f4get(v, e)); }
 
 // FIXED: Q5.27 values (the ring and the buffers hold int32 codes).
@@ -139,7 +148,7 @@ template <bool FIXED, bool PADDED, bool USIGN, bool BCAST, bool TRACK, int MAXC,
 __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
     const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_v0_tile,
     float *__restrict__ vout, const float *__restrict__ tab, const int32_t *__restrict__ qw,
-    const float *__restrict__ v0xy, const void *__restrict__ k4tab, HjLoop *lp, int sel, HjFlags *flags,
+    const float *__restrict__ v0xy, const void *__restrict__ k4tab, HjLoop *loop, int sel, HjFlags *flags,
     const HjGeom g, const TiledParams P)
 {
     static_assert(RPT == 1 || ((RPT == 2 || RPT == 4) && BCAST && USIGN && !FIXED && !PADDED),
@@ -167,15 +176,22 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
+    // An earlier step of the call that timed out ends the queued ones: the producer
+    // stops behind its first copy and sets the consumers' deadline to the past.
+    // Read here, the flag costs no time (behind the wait below, or tested by the
+    // consumers, steps of 15 us took 0.2 to 0.4 more); the step right behind the
+    // one that times out may still miss it and runs into its own deadline.
+    const int stop = !TRACK && tid == P.nconsumer ? *(volatile const int *)&loop->stop : 0;
     // Launched as a programmatic dependent of the previous step (the host sets
     // the launch attribute): everything above overlaps that step's end; from
     // here on the previous grid has completed and its V_n is visible.  Then
     // the next step may be scheduled as SMs free up (its CTAs wait here in
     // turn).  Without such a prerequisite both are no-ops.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (TRACK && lp->done) return;  // uniform across the grid
+    // uniform across the grid: converged, or an earlier step of the call timed out
+    if (TRACK && (loop->done | *(volatile const int *)&loop->stop)) return;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const float dt = (float)lp->dt[sel];
+    const float dt = (float)loop->dt[sel];
 
     // convergence mode (Algorithm 2's epsilon): this thread's largest |V_{n+1} - V_n|
     float dmf = 0.f;
@@ -214,6 +230,11 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
                     if (interior) tma_load_4d(dst + P.halo_floats, &map_v0_tile, &full[slot], 0, it.v0, it.y0, p);
                     used_mask |= 1u << slot;
                     last_phase = (last_phase & ~(1u << slot)) | (phase << slot);
+                    if (stop) {  // (the consumers need two planes to store anything)
+                        *(volatile unsigned long long *)deadline_p = 0ull;
+                        ok = false;
+                        break;
+                    }
                     ++issued;
                     if (++slot == P.stages) {
                         slot = 0;
@@ -222,14 +243,14 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
                 }
             }
             if (!ok) {
-                *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
+                step_timed_out(flags, loop);
                 *abort_flag = 1;
             }
             // drain: every copy this CTA issued must land before the CTA exits
             const unsigned long long drain_deadline = global_ns() + HJ_WAIT_NS;
             for (int s = 0; s < P.stages; ++s)
                 if (((used_mask >> s) & 1u) && !mbar_wait(&full[s], (last_phase >> s) & 1u, drain_deadline))
-                    *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
+                    step_timed_out(flags, loop);
         }
     } else {
         // ------------------------------------------------------------ consumers
@@ -660,13 +681,13 @@ __global__ void __launch_bounds__(MAXC + 32, 1) hj_step_tiled_kernel(
 #undef HJ_WAIT_NEXT
 #undef HJ_RELEASE_OLDEST
         if (!ok) {
-            *(volatile int *)&flags->status = HJ_ERR_TIMEOUT;
+            step_timed_out(flags, loop);
             *abort_flag = 1;
         }
     }
     if constexpr (TRACK) {
         __syncthreads();
-        hj_track_epilogue(lp, FIXED ? hj_abits((double)dmq * (1.0 / HJ_Q527_SCALE)) : hj_abits((double)dmf), scratch);
+        hj_track_epilogue(loop, FIXED ? hj_abits((double)dmq * (1.0 / HJ_Q527_SCALE)) : hj_abits((double)dmf), scratch);
     }
 }
 

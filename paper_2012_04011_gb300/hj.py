@@ -163,6 +163,8 @@ _SIGS = {
     "hj_barrier_selftest": (ctypes.c_int, [ctypes.c_int64, ctypes.POINTER(ctypes.c_int32),
                                            ctypes.POINTER(ctypes.c_int64)]),
     "hj_launch_selftest": (ctypes.c_int, [_VP, ctypes.c_int64]),
+    "hj_stop_selftest": (ctypes.c_int, [_VP, ctypes.c_double, ctypes.c_double, ctypes.c_double,
+                                        ctypes.POINTER(ctypes.c_int32)]),
     "hj_fp64_fma_probe": (ctypes.c_int, [ctypes.c_int64, ctypes.c_int32, _VP, ctypes.POINTER(ctypes.c_int64)]),
     "hj_read_value": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_double), ctypes.c_size_t]),
     "hj_read_value_device": (ctypes.c_int, [_VP, _VP, ctypes.c_int, ctypes.c_size_t]),
@@ -378,6 +380,15 @@ def hj_barrier_selftest(limit_ns: int):
 def hj_launch_selftest(g, launch: int):
     """Makes step launch number `launch` (1, 2, ...; 0: none) from here fail on the host."""
     _check(lib.hj_launch_selftest(g, int(launch)))
+
+
+def hj_stop_selftest(g, T: float, cfl: float = 0.8, threshold: float = 0.0):
+    """(status, stored) of a solve whose first step finds an earlier one timed out."""
+    stored = ctypes.c_int32(-1)
+    st = lib.hj_stop_selftest(g, float(T), float(cfl), float(threshold), ctypes.byref(stored))
+    if st != HJ_ERR_TIMEOUT:
+        _check(st)
+    return int(st), int(stored.value)
 
 
 def hj_read_value(g, out: np.ndarray | None = None, shape=None) -> np.ndarray:

@@ -1,6 +1,7 @@
 """Calls that fail leave a grid as it was, or say that its value is gone: a
 call on a stream that is being captured, a step launch that fails (on the
-host: no kernel of it runs)."""
+host: no kernel of it runs), a step that timed out (only the flags such a step
+leaves; no wait runs out)."""
 import numpy as np
 import pytest
 
@@ -124,3 +125,42 @@ def test_failed_autotune_leaves_the_grid_ready(hj):
         g.set_initial_value(V0)
         g.solve_brt(w.T, w.cfl)
         assert np.array_equal(g.read_value(), V)
+
+
+@pytest.mark.parametrize("prec", ["FP32", "Q527"])
+@pytest.mark.parametrize("xy", [False, True])
+@pytest.mark.parametrize("threshold", [0.0, 1e-3])
+@pytest.mark.parametrize("n", [(31, 31, 11, 16), (12, 10, 9, 33)])
+def test_steps_behind_a_timed_out_one_leave_at_once(hj, prec, xy, threshold, n):
+    w = scenes.custom_workload(n, n_circles=3, T=0.4, seed=sum(n))
+    V0 = scenes.initial_value(w.grid, w.scene)
+    out = []
+    with hj.Grid.for_workload(w, getattr(hj, "HJ_" + prec)) as g:
+        g.set_kernel(hj.HJ_KERNEL_TILED)
+        for _ in range(2):
+            if xy:
+                g.set_initial_value_xy(scenes.signed_distance_xy(w.grid, w.scene))
+            else:
+                g.set_initial_value(V0)
+            if not out:
+                assert hj.hj_stop_selftest(g.handle, w.T, w.cfl, threshold) == (hj.HJ_ERR_TIMEOUT, 0)
+                # the value is gone and the status stays until the next V0
+                assert not g.info().has_value
+                with pytest.raises(hj.HjError) as e:
+                    g.read_value()
+                assert e.value.status == hj.HJ_ERR_STATE
+                with pytest.raises(hj.HjError) as e:
+                    g.solve_brt(w.T, w.cfl)
+                assert e.value.status == hj.HJ_ERR_TIMEOUT
+                if xy:
+                    g.set_initial_value_xy(scenes.signed_distance_xy(w.grid, w.scene))
+                else:
+                    g.set_initial_value(V0)
+            g.solve_brt(w.T, w.cfl)
+            out.append(g.read_value())
+    assert np.array_equal(out[0], out[1])
+    with hj.Grid.for_workload(w, getattr(hj, "HJ_" + prec)) as g:
+        g.set_kernel(hj.HJ_KERNEL_TILED)
+        g.set_initial_value(V0)
+        g.solve_brt(w.T, w.cfl)
+        assert np.array_equal(g.read_value(), out[0])
