@@ -279,7 +279,10 @@ HJ_API hj_status hj_set_kernel(hj_grid *g, hj_kernel kernel);
 /* Tile shape of the tiled kernel: shape = {rows along y, rows along v, x
  * planes per work item, shared-memory stages}; a 0 entry is chosen
  * automatically.  HJ_ERR_UNSUPPORTED if the grid has no tiled kernel or the
- * shape does not fit (the previous shape then stays). */
+ * shape does not fit (the previous shape then stays).  Where V0 depends on (x,
+ * y) only, the kernel reads it from its field, and larger shapes fit; a shape
+ * that fits one form only leaves the other its automatic choice (of the stages
+ * first). */
 HJ_API hj_status hj_set_tile_shape(hj_grid *g, const int32_t shape[4]);
 
 /* Autotune the tiled kernel: time steps_per_trial (>= 1) step launches for
@@ -288,7 +291,8 @@ HJ_API hj_status hj_set_tile_shape(hj_grid *g, const int32_t shape[4]);
  * fastest of those.  Must be called right
  * after hj_set_initial_value[_device] (no step taken yet): trial steps read
  * V0 and write only the ping-pong buffers, and the time-loop state is put
- * back afterwards, so the next solve is unchanged.  results (may be NULL)
+ * back afterwards, so the next solve is unchanged.  The shape found is kept
+ * for V0s of the same form (one value per (x, y) or not).  results (may be NULL)
  * receives up to max_results candidates in the order tried, *nresults (may
  * be NULL) their count.  HJ_ERR_UNSUPPORTED without a tiled kernel,
  * HJ_ERR_STATE after a step. */

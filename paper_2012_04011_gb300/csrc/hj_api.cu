@@ -683,6 +683,29 @@ void hj_destroy_grid(hj_grid *g)
     free_grid(g);
 }
 
+// Sets up the tiled kernel with the shape requested for the current form of
+// V0.  A shape need only fit one of the two forms (a stage without V0 boxes is
+// smaller, its tiles and stage counts larger): where it does not fit the
+// current one, its stage count and then all of it is chosen automatically, so
+// that a grid the kernel takes never loses it to a V0.
+static bool setup_tiled(hj_grid *g)
+{
+    char why[160];
+    int32_t *req = g->tile_req[g->v0_bcast], keep[4];
+    memcpy(keep, req, sizeof(keep));
+    bool ok = hj_tiled_setup(g, why, sizeof(why));
+    if (!ok && keep[3] > 0) {
+        req[3] = 0;
+        ok = hj_tiled_setup(g, why, sizeof(why));
+    }
+    if (!ok && (keep[0] > 0 || keep[1] > 0 || keep[2] > 0)) {
+        memset(req, 0, sizeof(keep));
+        ok = hj_tiled_setup(g, why, sizeof(why));
+    }
+    memcpy(req, keep, sizeof(keep));
+    return ok;
+}
+
 hj_status hj_set_dynamics(hj_grid *g, hj_dynamics kind, const double *params, int32_t nparams)
 {
     g_err[0] = 0;
@@ -746,23 +769,21 @@ hj_status hj_set_dynamics(hj_grid *g, hj_dynamics kind, const double *params, in
     // prologue rebuilds the dt-scaled tables
     g->up_dt[0] = g->up_dt[1] = -1.0;
     g->has_dyn = true;
-    char why[160];
-    g->tiled_ok = hj_tiled_setup(g, why, sizeof(why));
+    g->tiled_ok = setup_tiled(g);
     if (g->kernel_req == HJ_KERNEL_TILED && !g->tiled_ok) g->kernel_req = HJ_KERNEL_AUTO;
     hj_onchip_setup(g);
     // a previously set V0 stays; the next solve continues with the new dynamics
     return HJ_OK;
 }
 
-// The tiled kernel's stage layout depends on whether V0 is broadcast from the
-// (x, y) field; redo its setup when that changes.
+// The tiled kernel's stage layout and the shape requested for it depend on
+// whether V0 is read from the (x, y) field; redo its setup when that changes.
 static void set_v0_mode(hj_grid *g, bool bcast)
 {
     if (g->v0_bcast == bcast) return;
     g->v0_bcast = bcast;
     if (g->has_dyn) {
-        char why[160];
-        g->tiled_ok = hj_tiled_setup(g, why, sizeof(why));
+        g->tiled_ok = setup_tiled(g);
         if (g->kernel_req == HJ_KERNEL_TILED && !g->tiled_ok) g->kernel_req = HJ_KERNEL_AUTO;
     }
 }
@@ -1275,13 +1296,22 @@ hj_status hj_set_tile_shape(hj_grid *g, const int32_t shape[4])
     if (!g->tiled_ok) return set_err(HJ_ERR_UNSUPPORTED, "this grid has no tiled kernel");
     if ((s = activate(g)) != HJ_OK) return s;
     HJ_CUDA(cudaStreamSynchronize(g->stream));
-    int32_t old[4];
+    int32_t old[2][4];
     memcpy(old, g->tile_req, sizeof(old));
-    memcpy(g->tile_req, shape, sizeof(old));
-    char why[160];
-    if (!hj_tiled_setup(g, why, sizeof(why))) {
+    for (int i = 0; i < 2; ++i) memcpy(g->tile_req[i], shape, sizeof(old[i]));
+    char why[160], why_field[160];
+    bool ok = hj_tiled_setup(g, why, sizeof(why));
+    if (!ok && !g->v0_bcast && check_flat(g)) {
+        // a 4D V0 of this grid may take the field form, and hj_autotune then finds
+        // shapes that fit only that: accepted before V0 is known, too
+        g->v0_bcast = true;
+        ok = hj_tiled_setup(g, why_field, sizeof(why_field));
+        g->v0_bcast = false;
+        ok = ok && setup_tiled(g);
+    }
+    if (!ok) {
         memcpy(g->tile_req, old, sizeof(old));
-        hj_tiled_setup(g, why, sizeof(why));
+        setup_tiled(g);
         return set_err(HJ_ERR_UNSUPPORTED, "tile shape rejected: %s", why);
     }
     return HJ_OK;
@@ -1304,7 +1334,8 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
     if (!cfl_step(g, 0.8, &dt_trial)) return set_err(HJ_ERR_UNSTABLE, "the CFL step is not a usable number");
     const int status0 = read_status(g);
     int32_t keep[4];
-    memcpy(keep, g->tile_req, sizeof(keep));
+    int32_t *req = g->tile_req[g->v0_bcast];  // (the shape is the best one for this form of V0)
+    memcpy(keep, req, sizeof(keep));
 
     // candidate (ty, tv): one consumer thread per (row, theta quad), at least
     // 8 warps; the 4 shapes with the fewest halo reads per row from each
@@ -1362,10 +1393,10 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
     for (int c = 0; c < nc; ++c) {
         int auto_xc = -1;
         for (int xc_mode = 0; xc_mode < 2; ++xc_mode) {
-            g->tile_req[0] = cands[c].ty;
-            g->tile_req[1] = cands[c].tv;
-            g->tile_req[2] = xc_mode == 0 ? 0 : g->n[0];  // automatic chunks, or one chunk per column
-            g->tile_req[3] = 0;
+            req[0] = cands[c].ty;
+            req[1] = cands[c].tv;
+            req[2] = xc_mode == 0 ? 0 : g->n[0];  // automatic chunks, or one chunk per column
+            req[3] = 0;
             if (!hj_tiled_setup(g, why, sizeof(why))) continue;
             if (xc_mode == 0) auto_xc = g->tile_xc;
             else if (g->tile_xc == auto_xc) continue;  // the automatic choice already was one chunk
@@ -1416,7 +1447,7 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
                 }
         best = 1e300;
         for (int r = 0; r < 3 && r < m; ++r) {
-            memcpy(g->tile_req, results[order[r]].shape, sizeof(g->tile_req));
+            memcpy(req, results[order[r]].shape, sizeof(keep));
             if (!hj_tiled_setup(g, why, sizeof(why))) continue;
             if ((s = run_steps(2)) != HJ_OK) break;
             if ((s = run_steps(3 * steps_per_trial)) != HJ_OK) break;
@@ -1437,18 +1468,20 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
         g->hflags->status = status0;
     }
     // keep the winner (or the previous shape if nothing ran)
-    if (best < 1e300)
-        memcpy(g->tile_req, best_req, sizeof(best_req));
-    else
-        memcpy(g->tile_req, keep, sizeof(keep));
-    if (!hj_tiled_setup(g, why, sizeof(why)) && s == HJ_OK)
-        s = set_err(HJ_ERR_CUDA, "autotune: the chosen tile shape (%d, %d, %d, %d) was rejected: %s", g->tile_req[0],
-                    g->tile_req[1], g->tile_req[2], g->tile_req[3], why);
-    else if (s == HJ_OK && best < 1e300 &&
-             (g->tile_ty != best_req[0] || g->tile_tv != best_req[1] || g->tile_xc != best_req[2] ||
-              g->tile_stages != best_req[3]))
-        s = set_err(HJ_ERR_CUDA, "autotune: tile shape (%d, %d, %d, %d) came out as (%d, %d, %d, %d)", best_req[0],
-                    best_req[1], best_req[2], best_req[3], g->tile_ty, g->tile_tv, g->tile_xc, g->tile_stages);
+    if (best < 1e300) {
+        memcpy(req, best_req, sizeof(best_req));
+        const bool ok = hj_tiled_setup(g, why, sizeof(why));
+        if (!ok && s == HJ_OK)
+            s = set_err(HJ_ERR_CUDA, "autotune: the chosen tile shape (%d, %d, %d, %d) was rejected: %s", req[0],
+                        req[1], req[2], req[3], why);
+        else if (s == HJ_OK && (g->tile_ty != best_req[0] || g->tile_tv != best_req[1] || g->tile_xc != best_req[2] ||
+                                g->tile_stages != best_req[3]))
+            s = set_err(HJ_ERR_CUDA, "autotune: tile shape (%d, %d, %d, %d) came out as (%d, %d, %d, %d)", best_req[0],
+                        best_req[1], best_req[2], best_req[3], g->tile_ty, g->tile_tv, g->tile_xc, g->tile_stages);
+    } else {
+        memcpy(req, keep, sizeof(keep));
+        setup_tiled(g);
+    }
     if (nresults) *nresults = count;
     return s;
 }

@@ -154,7 +154,8 @@ struct hj_grid {
     hj_kernel kernel_req;  // requested by hj_set_kernel
     bool tiled_ok;         // the tiled kernel supports this grid
     CUtensorMap tmap[4];   // V0, buffer A, buffer B with the halo box; V0 with the tile box (tiled kernel)
-    int32_t tile_req[4];   // requested (ty, tv, xc, stages); 0 = choose automatically
+    int32_t tile_req[2][4];  // requested (ty, tv, xc, stages) with V0 as boxes [0] and as a field [1] (v0_bcast);
+                             // 0 = choose automatically
     int32_t tile_ty, tile_tv, tile_xc, tile_stages;
     int32_t tiled_ctas, tiled_per_sm;
     bool tiled_usign;      // FP32: every theta quad has one sign of cos and of sin, and every speed is >= 0

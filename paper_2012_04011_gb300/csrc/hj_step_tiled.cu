@@ -270,7 +270,8 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
     // stages as fit; hj_autotune measures the candidates instead.
     const int q4 = g->p4 / 4;
     if (max_consumers(fixed) / q4 < 1) return fail("theta rows too long for one CTA");
-    int ty = g->tile_req[0], tv = g->tile_req[1];
+    const int32_t *req = g->tile_req[g->v0_bcast];
+    int ty = req[0], tv = req[1];
     if (ty <= 0 || tv <= 0) {
         const int cap = hj_tiled_variant(fixed, 2);
         double best = 1e300;
@@ -284,7 +285,7 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
                 const bool thin = fixed && ((a < 3 && g->n[1] > 2) || (b < 3 && g->n[2] > 2));
                 const bool fits = !thin && C.nconsumer <= cap && 4 * (size_t)C.stage_bytes + 2048 <= (size_t)maxsmem;
                 if (!fits && !(a == 1 && b == 1)) continue;
-                const double c = fits ? step_cost(g, C, sms > 0 ? sms : 1, g->tile_req[2]) : 1e299;
+                const double c = fits ? step_cost(g, C, sms > 0 ? sms : 1, req[2]) : 1e299;
                 if (c < best) {
                     best = c;
                     bty = a;
@@ -298,7 +299,7 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
     if (ty > g->n[1]) ty = g->n[1];
     while (consumers_of(g, ty, tv) > max_consumers(fixed) && ty > 1) --ty;
     while (consumers_of(g, ty, tv) > max_consumers(fixed) && tv > 1) --tv;
-    int stages = g->tile_req[3];
+    int stages = req[3];
     if (stages <= 0) {  // as many as fit in shared memory, up to MAX_STAGES
         TiledParams P1 = make_params(g, ty, tv, 1, 0);
         stages = (int)((maxsmem - 2048) / P1.stage_bytes);
@@ -320,7 +321,7 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
         per_sm < 1)
         return fail("tile shape does not fit on an SM");
     const int slots = sms * per_sm;
-    const int xc = g->tile_req[2] > 0 ? g->tile_req[2] : best_chunk(g, P.ncol, slots);
+    const int xc = req[2] > 0 ? req[2] : best_chunk(g, P.ncol, slots);
     P = make_params(g, ty, tv, stages, xc);
 
     // tensor maps, dims (p4, n3, n2, n1): V0 / buffer A / buffer B with the

@@ -183,3 +183,56 @@ def test_flat_4d_v0_is_recognised_and_one_odd_cell_is_not_lost(hj):
     far = np.ones(V0.shape, bool)
     far[27:34, 17:24, 37:44, 47:54] = False  # three steps reach three cells
     assert np.array_equal(outs[2][far], outs[1][far])
+
+
+def test_tile_of_one_v0_form_does_not_cost_the_other_the_tiled_kernel(hj):
+    """A tile found (or set) with a flat 4D V0 need not fit with V0 boxes: the
+    tiled kernel stays for a V0 that varies within a column, with a shape that
+    fits, the flat form's shape is there again for the next flat V0, and a new
+    grid accepts it before its V0 is known."""
+    import torch
+    w = scenes.custom_workload((64, 64, 48, 96), n_circles=4, T=0.05, seed=5)
+    V0 = scenes.initial_value(w.grid, w.scene).astype(np.float32)
+    odd = V0.copy()
+    odd[30, 20, 40, 50] -= 0.5
+    flat, odd = torch.from_numpy(V0).cuda(), torch.from_numpy(odd).cuda()
+
+    def solve_to_end(g, v0):
+        g.set_initial_value(v0)
+        st = g.solve_brt(w.T, w.cfl)
+        assert st.kernel == g.info().kernel == hj.HJ_KERNEL_TILED
+        out = torch.empty(V0.shape, dtype=torch.float32, device="cuda")
+        return g.read_value_device(out).cpu().numpy(), list(g.info().tile)
+
+    with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+        g.set_kernel(hj.HJ_KERNEL_TILED)
+        ref_odd, tile_odd = solve_to_end(g, odd)
+        ref_flat, _ = solve_to_end(g, flat)
+    # 8 stages of a 4 x 8 tile: 146 KB without V0 boxes, 283 KB with them
+    for shape in (None, [4, 8, 32, 8]):
+        with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+            g.set_kernel(hj.HJ_KERNEL_TILED)
+            g.set_initial_value(flat)
+            if shape is None:
+                g.autotune(2)
+            else:
+                g.set_tile_shape(shape)
+            best = list(g.info().tile)
+            assert shape is None or best == shape
+            got, tile = solve_to_end(g, odd)
+            assert np.array_equal(got, ref_odd)
+            assert shape is not None or tile == tile_odd  # what was tuned is the other form
+            got, tile = solve_to_end(g, flat)
+            assert tile == best and np.array_equal(got, ref_flat)
+        with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+            g.set_kernel(hj.HJ_KERNEL_TILED)
+            g.set_tile_shape(best)
+            got, tile = solve_to_end(g, flat)
+            assert tile == best and np.array_equal(got, ref_flat)
+            g.set_dynamics(hj.HJ_DYN_CAR4D, (w.a_max, w.w_max))
+            assert list(g.info().tile) == best
+            assert np.array_equal(solve_to_end(g, odd)[0], ref_odd)
+        with pytest.raises(hj.HjError) as e:  # fits neither form
+            with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+                g.set_tile_shape([16, 16, 32, 8])
+        assert e.value.status == hj.HJ_ERR_UNSUPPORTED
