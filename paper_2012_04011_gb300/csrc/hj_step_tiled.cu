@@ -281,8 +281,9 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
                 if ((ty > 0 && a != ty) || (tv > 0 && b != tv)) continue;
                 const TiledParams C = make_params(g, a, b, 1, 0);
                 // (fixed point: tiles of one or two rows along an axis measured slower
-                // than the estimate, 70x90x40x72 69 us at 15 x 2, 61 at 6 x 5)
-                const bool thin = fixed && ((a < 3 && g->n[1] > 2) || (b < 3 && g->n[2] > 2));
+                // than the estimate, 70x90x40x72 69 us at 15 x 2, 61 at 6 x 5; an extent
+                // that is requested is taken as it is)
+                const bool thin = fixed && ((ty <= 0 && a < 3) || (tv <= 0 && b < 3));
                 const bool fits = !thin && C.nconsumer <= cap && 4 * (size_t)C.stage_bytes + 2048 <= (size_t)maxsmem;
                 if (!fits && !(a == 1 && b == 1)) continue;
                 const double c = fits ? step_cost(g, C, sms > 0 ? sms : 1, req[2]) : 1e299;

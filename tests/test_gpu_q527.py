@@ -233,3 +233,28 @@ def test_q527_items_over_several_rounds(hj, shape):
         st_t = g.solve_brt(w.T, w.cfl)
         assert st_t.kernel == hj.HJ_KERNEL_TILED and st_t.steps == st.steps
         assert np.array_equal(read_codes(g), Q)
+
+
+@pytest.mark.parametrize("prec", ["FP32", "Q527"])
+@pytest.mark.parametrize("axis", [0, 1])
+def test_tile_shape_given_along_one_axis_is_kept(hj, prec, axis):
+    """A request for the rows along y or along v only: that extent is taken, the
+    other one chosen, down to tiles of one row (which the automatic choice leaves
+    out in fixed point), with the same codes."""
+    w = scenes.workload("car4d_31x31x11x16")
+    V0 = scenes.initial_value(w.grid, w.scene)
+    ref = None
+    with hj.Grid.for_workload(w, getattr(hj, "HJ_" + prec)) as g:
+        g.set_kernel(hj.HJ_KERNEL_TILED)
+        for rows in (0, 1, 2, 3, 5):
+            shape = [0, 0, 0, 0]
+            shape[axis] = rows
+            g.set_tile_shape(shape)
+            tile = list(g.info().tile)
+            if rows:
+                assert tile[axis] == rows and tile[1 - axis] > 1, tile
+            g.set_initial_value(V0)
+            g.solve_brt(w.T, w.cfl)
+            V = g.read_value()
+            ref = V if ref is None else ref
+            assert np.array_equal(V, ref), tile
