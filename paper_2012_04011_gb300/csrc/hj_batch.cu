@@ -964,7 +964,8 @@ hj_status rebuild(hj_batch *b)
         b->bp = bp;
         BatchKernelFn fn = batch_kernel(bp.nconsumer);
         const size_t smem = batch_smem(bp);
-        HJB_CUDA(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        // (the largest: the limit is the kernel's, which other batches share)
+        HJB_CUDA(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, b->maxsmem));
         int per_sm = 0;
         HJB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, bp.nconsumer + 32, smem));
         if (per_sm < 1) return bfail(HJ_ERR_UNSUPPORTED, "batch kernel shape does not fit on an SM");

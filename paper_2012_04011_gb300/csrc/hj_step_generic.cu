@@ -871,7 +871,8 @@ cudaError_t launch_resident(hj_grid *g, long long n, long long k, bool cut)
 {
     const void *fn = (const void *)hj_step_resident_kernel<T, TRACK>;
     const size_t smem = resident_table_bytes(g);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the largest: another thread's grid may set the limit between here and the launch)
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RES_MAX_TABLE);
     if (e != cudaSuccess) return e;
     int sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);

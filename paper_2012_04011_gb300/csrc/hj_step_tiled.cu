@@ -314,8 +314,10 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
     const void *fn = (const void *)kernel_fn(fixed, g->p4 != g->n[3], usign, g->v0_bcast, false, P.nconsumer, P.rpt);
     const void *fn_track =
         (const void *)kernel_fn(fixed, g->p4 != g->n[3], usign, g->v0_bcast, true, P.nconsumer, P.rpt);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(fn_track, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    // (the limit belongs to the kernel, not to the grid: always the largest, so that
+    // a grid set up later with a smaller ring does not lower it under this one's)
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsmem) != cudaSuccess ||
+        cudaFuncSetAttribute(fn_track, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsmem) != cudaSuccess)
         return fail("cannot raise the shared-memory limit");
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, P.nconsumer + 32, smem) != cudaSuccess ||

@@ -275,3 +275,21 @@ def test_many_slots_set_in_one_call(hj):
         with pytest.raises(hj.HjError) as e:  # a count that does not match the slot's grid
             b.set_initial_values(slots[:1], [v0s[1]])
         assert e.value.status == hj.HJ_ERR_INVALID_ARG
+
+
+def test_a_later_batch_does_not_lower_the_shared_memory_limit(hj):
+    """Two batches on the same batch kernel (480 consumers: tiles of 6 x 5 rows
+    of 64 points and of 8 x 15 rows of 16), the second with a smaller ring: the
+    kernel's shared-memory limit is one for both, and the first, laid out
+    already, must still launch."""
+    ws = [scenes.custom_workload(n, n_circles=3, T=0.2, seed=7) for n in ((20, 48, 20, 64), (12, 8, 15, 16))]
+    v0s = [scenes.initial_value(w.grid, w.scene) for w in ws]
+    with hj.Batch(1) as a, hj.Batch(1) as b:
+        for bt, w in ((a, ws[0]), (b, ws[1])):
+            bt.add_workload(w)
+        for k in (0, 1, 0):
+            bt = (a, b)[k]
+            bt.set_initial_value(0, v0s[k])
+            bt.set_horizon(0, ws[k].T, ws[k].cfl)
+            assert bt.advance().finished == 1
+            assert np.array_equal(bt.read_value(0), single_grid(hj, ws[k], v0s[k])[0])

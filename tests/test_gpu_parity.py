@@ -549,3 +549,23 @@ def test_negative_speeds_and_shifted_domain(hj, dyn):
             out = torch.empty(V0.size, dtype=torch.int32, device="cuda")
             gr.read_value_device(out)
         assert np.array_equal(out.cpu().numpy().reshape(g.n), Qo)
+
+
+def test_a_later_grid_does_not_lower_the_shared_memory_limit(hj):
+    """Two grids on one variant of the tiled kernel, the second with half the
+    ring: the kernel's shared-memory limit is one for both, and the first must
+    still launch."""
+    w = scenes.workload("car4d_31x31x11x16")
+    V0 = scenes.initial_value(w.grid, w.scene)
+    for prec in (hj.HJ_FP32, hj.HJ_Q527):
+        with hj.Grid.for_workload(w, prec) as a, hj.Grid.for_workload(w, prec) as b:
+            out = []
+            for g, stages in ((a, 8), (b, 4)):
+                g.set_kernel(hj.HJ_KERNEL_TILED)
+                g.set_tile_shape([12, 10, 0, stages])
+                assert list(g.info().tile)[:2] == [12, 10] and g.info().tile[3] == stages
+                g.set_initial_value(V0)
+            for g in (a, b):
+                g.solve_brt(w.T, w.cfl)
+                out.append(g.read_value())
+            assert np.array_equal(out[0], out[1])
