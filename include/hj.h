@@ -387,7 +387,9 @@ HJ_API size_t hj_batch_slot_bytes(const int32_t n[4]);
 HJ_API hj_status hj_batch_add(hj_batch *b, const int32_t n[4], const double lo[4], const double hi[4],
                               const double params[2], int32_t *slot);
 
-/* Free a slot (its device memory returns to the budget). */
+/* Free a slot.  Its device memory returns to the budget; the batch keeps up
+ * to 1 GiB of such memory, the latest freed, for new slots of the same sizes,
+ * until it is destroyed or another allocation of this library needs it. */
 HJ_API hj_status hj_batch_remove(hj_batch *b, int32_t slot);
 
 /* V0 of a slot from a host FP64 array or a device FP32/FP64 array (layout as

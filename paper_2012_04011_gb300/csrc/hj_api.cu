@@ -643,21 +643,21 @@ hj_status hj_create_grid(const int32_t n[4], const double lo[4], const double hi
     }
     size_t arr = (size_t)g->nint * g->esize;
     size_t ncoef = (size_t)n[2] * n[3];
-    if (e == cudaSuccess) e = cudaMalloc(&g->v0, arr);
-    if (e == cudaSuccess) e = cudaMalloc(&g->buf, 2 * arr);
+    if (e == cudaSuccess) e = hj_malloc((void **)&g->v0, arr);
+    if (e == cudaSuccess) e = hj_malloc((void **)&g->buf, 2 * arr);
     // FP64 coefficients for FP64 and Q5.27 grids (alpha^max and dt are FP64)
     const size_t coef_bytes = ncoef * (prec == HJ_FP32 ? sizeof(HjCoef<float>) : sizeof(HjCoef<double>));
     const size_t qw_bytes = prec == HJ_Q527 ? 2 * sizeof(int32_t) * hj_qw_count(n[2], g->p4) : 0;
     const size_t scaled_bytes = prec == HJ_FP64 ? 2 * sizeof(double) * hj_scaled_count(n[2], g->p4) : 0;
     const size_t k4_bytes = (size_t)n[2] * (prec == HJ_FP32 ? 2 * sizeof(float) : sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&g->coef, coef_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&g->tab_tiled, sizeof(float) * ((size_t)n[2] + 3 * (size_t)g->p4));
-    if (e == cudaSuccess && prec == HJ_FP64) e = cudaMalloc(&g->scaled, scaled_bytes);
-    if (e == cudaSuccess && prec == HJ_Q527) e = cudaMalloc(&g->qw, qw_bytes);
+    if (e == cudaSuccess) e = hj_malloc((void **)&g->coef, coef_bytes);
+    if (e == cudaSuccess) e = hj_malloc((void **)&g->tab_tiled, sizeof(float) * ((size_t)n[2] + 3 * (size_t)g->p4));
+    if (e == cudaSuccess && prec == HJ_FP64) e = hj_malloc((void **)&g->scaled, scaled_bytes);
+    if (e == cudaSuccess && prec == HJ_Q527) e = hj_malloc((void **)&g->qw, qw_bytes);
     const size_t xy_bytes = (size_t)n[0] * n[1] * g->esize;
-    if (e == cudaSuccess) e = cudaMalloc(&g->v0xy, xy_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&g->k4tab, k4_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&g->loop, sizeof(HjLoop));
+    if (e == cudaSuccess) e = hj_malloc((void **)&g->v0xy, xy_bytes);
+    if (e == cudaSuccess) e = hj_malloc((void **)&g->k4tab, k4_bytes);
+    if (e == cudaSuccess) e = hj_malloc((void **)&g->loop, sizeof(HjLoop));
     if (e == cudaSuccess) e = cudaHostAlloc(&g->hloop, sizeof(HjLoop), cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaHostAlloc(&g->hflags, sizeof(HjFlags), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&g->dflags, g->hflags, 0);

@@ -37,6 +37,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -641,7 +642,8 @@ struct hj_batch {
     size_t budget = 0, used_bytes = 0;
     // device memory of removed slots, kept for the next ones of the same size (a
     // served request costs an allocation and a free otherwise): at most
-    // B_POOL_BYTES, and within the budget together with the slots in use
+    // B_POOL_BYTES, within the budget together with the slots in use, and given
+    // up when an allocation of the library finds the device out of memory
     std::vector<std::pair<void *, size_t>> pool;
     size_t pool_bytes = 0;
     cudaStream_t stream = nullptr;
@@ -701,42 +703,80 @@ hj_status bfail(hj_status s, const char *fmt, ...)
     } while (0)
 
 
-void release_pool(hj_batch *b)
+// Every batch that may keep memory of removed slots, and the lock of their
+// pools: an allocation on any thread that finds the device out of memory frees
+// them (hj_malloc).  Never destroyed: batches may outlive static objects.
+std::mutex &pool_mutex()
 {
-    for (auto &m : b->pool) cudaFree(m.first);
-    b->pool.clear();
-    b->pool_bytes = 0;
+    static std::mutex *m = new std::mutex;
+    return *m;
+}
+std::vector<hj_batch *> &pool_owners()
+{
+    static std::vector<hj_batch *> *v = new std::vector<hj_batch *>;
+    return *v;
+}
+
+// Frees the oldest kept blocks until at most `keep` bytes are left (the lock
+// is held; no queued work uses them).
+void shrink_pool(hj_batch *b, size_t keep)
+{
+    size_t k = 0;
+    for (; k < b->pool.size() && b->pool_bytes > keep; ++k) {
+        cudaFree(b->pool[k].first);
+        b->pool_bytes -= b->pool[k].second;
+    }
+    b->pool.erase(b->pool.begin(), b->pool.begin() + k);
 }
 
 // Device memory of a new slot: a kept block of that size, else a fresh one.
 cudaError_t slot_alloc(hj_batch *b, size_t bytes, void **mem)
 {
-    for (size_t i = 0; i < b->pool.size(); ++i)
-        if (b->pool[i].second == bytes) {
-            *mem = b->pool[i].first;
-            b->pool_bytes -= bytes;
-            b->pool.erase(b->pool.begin() + i);
-            return cudaSuccess;
-        }
-    if (b->used_bytes + b->pool_bytes + bytes > b->budget) release_pool(b);
-    cudaError_t e = cudaMalloc(mem, bytes);
-    if (e == cudaErrorMemoryAllocation && !b->pool.empty()) {
-        cudaGetLastError();
-        release_pool(b);
-        e = cudaMalloc(mem, bytes);
+    {
+        std::lock_guard<std::mutex> lock(pool_mutex());
+        for (size_t i = 0; i < b->pool.size(); ++i)
+            if (b->pool[i].second == bytes) {
+                *mem = b->pool[i].first;
+                b->pool_bytes -= bytes;
+                b->pool.erase(b->pool.begin() + i);
+                return cudaSuccess;
+            }
+        // (the caller has checked used_bytes + bytes against the budget)
+        shrink_pool(b, b->budget - b->used_bytes - bytes);
     }
-    return e;
+    return hj_malloc(mem, bytes);
 }
 
-// Memory of a removed slot (no longer in used_bytes; the stream is idle).
+// Memory of a removed slot (no longer in used_bytes; the stream is idle): kept
+// in place of the oldest blocks, so that the sizes served now are the ones
+// that find a block.
 void slot_free(hj_batch *b, void *mem, size_t bytes)
 {
-    if (b->used_bytes + b->pool_bytes + bytes > b->budget || b->pool_bytes + bytes > B_POOL_BYTES) {
+    std::lock_guard<std::mutex> lock(pool_mutex());
+    const size_t left = b->budget > b->used_bytes ? b->budget - b->used_bytes : 0;
+    const size_t cap = left < B_POOL_BYTES ? left : B_POOL_BYTES;
+    if (bytes > cap) {
         cudaFree(mem);
         return;
     }
+    shrink_pool(b, cap - bytes);
     b->pool.push_back({mem, bytes});
     b->pool_bytes += bytes;
+}
+
+// Frees what the batches on the current device keep; whether that was anything.
+bool release_pools()
+{
+    int device = -1;
+    if (cudaGetDevice(&device) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(pool_mutex());
+    bool any = false;
+    for (hj_batch *b : pool_owners()) {
+        if (b->device != device || b->pool.empty()) continue;
+        any = true;
+        shrink_pool(b, 0);
+    }
+    return any;
 }
 
 // Tile of one slot for a block of nc consumer threads (ty x tv <= nc / q4).
@@ -949,7 +989,7 @@ hj_status rebuild(hj_batch *b)
         b->d_items = nullptr;
         b->items_cap = 0;
         const int cap = need + (int)items.size();
-        HJB_CUDA(cudaMalloc(&b->d_items, sizeof(BatchItem) * cap));
+        HJB_CUDA(hj_malloc((void **)&b->d_items, sizeof(BatchItem) * cap));
         b->items_cap = cap;
     }
     HJB_CUDA(cudaStreamSynchronize(b->stream));
@@ -1110,6 +1150,16 @@ hj_status check_slot(const hj_batch *b, int slot)
 
 }  // namespace
 
+cudaError_t hj_malloc(void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && release_pools()) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 extern "C" {
 
 hj_status hj_batch_create(int32_t max_slots, size_t memory_budget, void *cuda_stream, hj_batch **out)
@@ -1127,6 +1177,7 @@ hj_status hj_batch_create(int32_t max_slots, size_t memory_budget, void *cuda_st
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&b->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, b->device);
     size_t free_b = 0, total_b = 0;
+    if (memory_budget == 0) release_pools();  // (what other batches keep counts as free)
     if (e == cudaSuccess) e = cudaMemGetInfo(&free_b, &total_b);
     b->budget = memory_budget > 0 ? memory_budget : (size_t)(0.9 * (double)free_b);
     if (e == cudaSuccess && cuda_stream) {
@@ -1135,16 +1186,16 @@ hj_status hj_batch_create(int32_t max_slots, size_t memory_budget, void *cuda_st
         e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
         b->own_stream = e == cudaSuccess;
     }
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_insts, sizeof(BatchInst) * max_slots);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_slots, sizeof(BatchSlot) * max_slots);
+    if (e == cudaSuccess) e = hj_malloc((void **)&b->d_insts, sizeof(BatchInst) * max_slots);
+    if (e == cudaSuccess) e = hj_malloc((void **)&b->d_slots, sizeof(BatchSlot) * max_slots);
     if (e == cudaSuccess) e = cudaHostAlloc(&b->h_slots, sizeof(BatchSlot) * max_slots, cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaHostAlloc(&b->h_setup, sizeof(SlotSetup) * max_slots, cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_setup, sizeof(SlotSetup) * max_slots);
+    if (e == cudaSuccess) e = hj_malloc((void **)&b->d_setup, sizeof(SlotSetup) * max_slots);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_setup, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_ctl, sizeof(BatchCtl));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_rounds, sizeof(int) * (B_MAX_ROUNDS + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_rounds_done, sizeof(int) * max_slots);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_maps, sizeof(CUtensorMap) * 4 * max_slots);
+    if (e == cudaSuccess) e = hj_malloc((void **)&b->d_ctl, sizeof(BatchCtl));
+    if (e == cudaSuccess) e = hj_malloc((void **)&b->d_rounds, sizeof(int) * (B_MAX_ROUNDS + 1));
+    if (e == cudaSuccess) e = hj_malloc((void **)&b->d_rounds_done, sizeof(int) * max_slots);
+    if (e == cudaSuccess) e = hj_malloc((void **)&b->d_maps, sizeof(CUtensorMap) * 4 * max_slots);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreate(&b->ev[i]);
     if (e == cudaSuccess && b->own_stream) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
     if (e == cudaSuccess) {
@@ -1161,6 +1212,10 @@ hj_status hj_batch_create(int32_t max_slots, size_t memory_budget, void *cuda_st
         hj_batch_destroy(b);
         return s;
     }
+    {
+        std::lock_guard<std::mutex> lock(pool_mutex());
+        pool_owners().push_back(b);
+    }
     *out = b;
     return HJ_OK;
 }
@@ -1171,7 +1226,12 @@ void hj_batch_destroy(hj_batch *b)
     if (b->stream) cudaStreamSynchronize(b->stream);
     for (auto &s : b->slots)
         if (s.mem) cudaFree(s.mem);
-    release_pool(b);
+    {
+        std::lock_guard<std::mutex> lock(pool_mutex());
+        std::vector<hj_batch *> &owners = pool_owners();
+        owners.erase(std::remove(owners.begin(), owners.end(), b), owners.end());
+        shrink_pool(b, 0);
+    }
     if (b->d_insts) cudaFree(b->d_insts);
     if (b->d_slots) cudaFree(b->d_slots);
     if (b->h_slots) cudaFreeHost(b->h_slots);

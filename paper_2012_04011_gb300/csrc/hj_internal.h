@@ -376,6 +376,10 @@ __device__ __forceinline__ int32_t hj_q527_update(int32_t vc, int32_t v0, long l
     return (int32_t)(vn < -2147483648LL ? -2147483648LL : vn);
 }
 
+// cudaMalloc; if the device is out of memory, once more after the batches have
+// freed the memory of removed slots that they keep (hj_batch.cu).
+cudaError_t hj_malloc(void **p, size_t bytes);
+
 // Batch internals for the server: pull all slot states once, then query the
 // host copy (done flag and step count of a slot).
 hj_status hj_batch_refresh(hj_batch *b);

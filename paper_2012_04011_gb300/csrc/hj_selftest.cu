@@ -94,7 +94,7 @@ hj_status run_selftest(int64_t limit_ns, int32_t *status, int64_t *waited_ns, Se
     }
     char *d = nullptr;
     const size_t bytes = 16 + sizeof(HjResidentSync);
-    cudaError_t e = cudaMalloc(&d, bytes);
+    cudaError_t e = hj_malloc((void **)&d, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();  // the failed allocation must not fail later launch checks
         hj_internal_set_error(cudaGetErrorString(e));

@@ -915,7 +915,7 @@ bool hj_resident_supported(const hj_grid *g)
 cudaError_t hj_launch_step_resident(hj_grid *g, long long n, long long k, bool cut)
 {
     if (!g->rsync) {
-        cudaError_t e = cudaMalloc(&g->rsync, sizeof(HjResidentSync));
+        cudaError_t e = hj_malloc((void **)&g->rsync, sizeof(HjResidentSync));
         if (e != cudaSuccess) {
             g->rsync = nullptr;
             return e;
