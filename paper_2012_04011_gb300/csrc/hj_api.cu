@@ -62,15 +62,13 @@ __device__ __forceinline__ T elem_from_f64(double x)
 }
 
 // Dense row-major [N1][N2][N3][N4] (any of double/float) -> internal layout
-// (rows padded to p4, pad lanes zero).  Flags non-finite input.  With nonflat
-// given, also flags a value that differs from the first one of its column (n3
-// rows) and stores those first values in xy.
+// (rows padded to p4, pad lanes zero).  Flags non-finite input.
 template <typename Tin, typename T>
 __global__ void ingest_kernel(const Tin *__restrict__ src, T *__restrict__ dst, int n4, int p4, long long nrows,
-                              int *nonfinite, int *nonflat = nullptr, int n3 = 1, T *xy = nullptr)
+                              int *nonfinite)
 {
     long long total = nrows * p4;
-    int bad = 0, varies = 0;
+    int bad = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
         long long row = i / p4;
@@ -80,17 +78,41 @@ __global__ void ingest_kernel(const Tin *__restrict__ src, T *__restrict__ dst, 
             double x = elem_to_f64<Tin>(src[row * n4 + l]);
             if (!isfinite(x)) bad = 1;
             v = elem_from_f64<T>(x);
-            if (nonflat) {  // (the sign of a zero counts)
-                const long long col = row / n3;
-                const T first = elem_from_f64<T>(elem_to_f64<Tin>(src[col * n3 * n4]));
-                if (v != first || signbit((double)v) != signbit((double)first)) varies = 1;
-                if (l == 0 && row == col * n3) xy[col] = v;
-            }
         }
         dst[i] = v;
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0) *(volatile int *)nonfinite = 1;
-    if (nonflat && __syncthreads_or(varies) && threadIdx.x == 0) *(volatile int *)nonflat = 1;
+}
+
+// The same for an FP32 grid without pad lanes, which also flags a value that
+// differs from the first one of its column (one (x, y): len values, contiguous
+// on both sides; the sign of a zero counts) and stores those first values in
+// xy.  A block takes whole columns, so that an index costs no division: bound
+// by HBM.  128x128x64x96 from FP32 (FP64) on the device, us per call: 760 (934)
+// with the check in the kernel above, 469 (516) there without it, 135 (375) so;
+// 16x16x256x256, few long columns, 59 (87) against 102 (111) without the check.
+template <typename Tin>
+__global__ void __launch_bounds__(256) ingest_flat_kernel(const Tin *__restrict__ src, float *__restrict__ dst,
+                                                          long long ncol, int len, float *__restrict__ xy,
+                                                          int *nonfinite, int *nonflat)
+{
+    int bad = 0, varies = 0;
+    for (long long col = blockIdx.x; col < ncol; col += gridDim.x) {
+        const Tin *in = src + col * len;
+        float *out = dst + col * len;
+        const float first = elem_from_f64<float>(elem_to_f64<Tin>(in[0]));
+        if (threadIdx.x == 0) xy[col] = first;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < len; i += 256) {
+            const double x = elem_to_f64<Tin>(in[i]);
+            if (!isfinite(x)) bad = 1;
+            const float v = elem_from_f64<float>(x);
+            if (__float_as_int(v) != __float_as_int(first)) varies = 1;
+            out[i] = v;
+        }
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) *(volatile int *)nonfinite = 1;
+    if (__syncthreads_or(varies) && threadIdx.x == 0) *(volatile int *)nonflat = 1;
 }
 
 // V0 that depends only on (x, y): an N1*N2 field replicated over v and theta
@@ -831,12 +853,18 @@ static hj_status ingest_4d(hj_grid *g, const void *src, hj_precision dtype)
     const long long nrows = (long long)g->n[0] * g->n[1] * g->n[2];
     const bool check = check_flat(g);
     with_elem(dtype, [&](auto ein) {
+        using Tin = decltype(ein);
+        if (check) {
+            const long long ncol = (long long)g->n[0] * g->n[1];
+            ingest_flat_kernel<Tin><<<grid_blocks(ncol, 1), 256, 0, g->stream>>>(
+                (const Tin *)src, (float *)g->v0, ncol, g->n[2] * g->n[3], (float *)g->v0xy, &g->dflags->nonfinite,
+                &g->dflags->nonflat);
+            return;
+        }
         with_elem(g->prec, [&](auto e) {
-            using Tin = decltype(ein);
             using T = decltype(e);
             ingest_kernel<Tin, T><<<grid_blocks(g->nint, 256), 256, 0, g->stream>>>(
-                (const Tin *)src, (T *)g->v0, g->n[3], g->p4, nrows, &g->dflags->nonfinite,
-                check ? &g->dflags->nonflat : nullptr, g->n[2], (T *)g->v0xy);
+                (const Tin *)src, (T *)g->v0, g->n[3], g->p4, nrows, &g->dflags->nonfinite);
         });
     });
     g->v0_xy = false;

@@ -236,3 +236,37 @@ def test_tile_of_one_v0_form_does_not_cost_the_other_the_tiled_kernel(hj):
             with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
                 g.set_tile_shape([16, 16, 32, 8])
         assert e.value.status == hj.HJ_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float64", "pinned"])
+def test_flat_check_sees_every_cell_of_a_column(hj, dtype):
+    """The ingest of a grid of at least 2^24 cells compares every value with the
+    first of its column: one changed value at the ends of the first and the last
+    column (and one beyond a block's first pass) keeps the V0 boxes, whose
+    tile has room for them; a NaN anywhere is refused."""
+    import torch
+    w = scenes.custom_workload((64, 65, 65, 64), n_circles=4, T=0.02, seed=5)
+    V0 = scenes.initial_value(w.grid, w.scene).astype(np.float64 if dtype == "float64" else np.float32)
+    flat = torch.from_numpy(V0)
+    with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+        def put(cell, value):
+            old = flat[cell].item() if cell else None
+            if cell:
+                flat[cell] = value
+            try:
+                g.set_initial_value(flat.double().pin_memory().numpy() if dtype == "pinned" else flat.cuda())
+            finally:
+                if cell:
+                    flat[cell] = old
+            g.advance_brt(w.T, w.cfl, 1)
+            out = torch.empty(V0.shape, dtype=torch.float32, device="cuda")
+            return g.read_value_device(out).cpu()
+        ref, field_tile = put(None, None), list(g.info().tile)
+        for cell in ((0, 0, 0, 0), (0, 0, 64, 63), (63, 64, 0, 0), (63, 64, 64, 63), (31, 32, 5, 3)):
+            got = put(cell, flat[cell].item() - 0.25)
+            assert list(g.info().tile) != field_tile
+            assert got[cell] <= ref[cell] - 0.2 and int((got != ref).sum()) < 20
+            assert torch.equal(put(None, None), ref) and list(g.info().tile) == field_tile
+            with pytest.raises(hj.HjError) as e:
+                put(cell, float("nan"))
+            assert e.value.status == hj.HJ_ERR_INVALID_ARG
