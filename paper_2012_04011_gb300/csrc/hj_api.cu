@@ -542,7 +542,6 @@ void free_grid(hj_grid *g)
     if (g->qw) cudaFree(g->qw);
     if (g->v0xy) cudaFree(g->v0xy);
     if (g->k4tab) cudaFree(g->k4tab);
-    if (g->rsync) cudaFree(g->rsync);
     if (g->loop) cudaFree(g->loop);
     if (g->hloop) cudaFreeHost(g->hloop);
     if (g->hflags) cudaFreeHost(g->hflags);
@@ -679,7 +678,11 @@ hj_status hj_create_grid(const int32_t n[4], const double lo[4], const double hi
     const size_t xy_bytes = (size_t)n[0] * n[1] * g->esize;
     if (e == cudaSuccess) e = hj_malloc((void **)&g->v0xy, xy_bytes);
     if (e == cudaSuccess) e = hj_malloc((void **)&g->k4tab, k4_bytes);
-    if (e == cudaSuccess) e = hj_malloc((void **)&g->loop, sizeof(HjLoop));
+    // the loop's constants and the cooperative kernels' flags in one allocation (the
+    // flags: allocated by the first solve they cost it up to 90 us, 31x31x11x16)
+    constexpr size_t loop_bytes = (sizeof(HjLoop) + 127) / 128 * 128;
+    if (e == cudaSuccess) e = hj_malloc((void **)&g->loop, loop_bytes + sizeof(HjResidentSync));
+    if (e == cudaSuccess) g->rsync = (HjResidentSync *)((char *)g->loop + loop_bytes);
     if (e == cudaSuccess) e = cudaHostAlloc(&g->hloop, sizeof(HjLoop), cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaHostAlloc(&g->hflags, sizeof(HjFlags), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&g->dflags, g->hflags, 0);
@@ -692,7 +695,8 @@ hj_status hj_create_grid(const int32_t n[4], const double lo[4], const double hi
         free_grid(g);
         return s;
     }
-    g->device_bytes = 3 * arr + coef_bytes + qw_bytes + scaled_bytes + xy_bytes + k4_bytes + sizeof(HjLoop);
+    g->device_bytes = 3 * arr + coef_bytes + qw_bytes + scaled_bytes + xy_bytes + k4_bytes + loop_bytes +
+                      sizeof(HjResidentSync);
     reset_state(g);
     *out = g;
     return HJ_OK;

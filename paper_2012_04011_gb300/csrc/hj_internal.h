@@ -74,7 +74,8 @@ struct HjScaledCoef {
 // the on-chip kernel has published.  Zeroed before every such launch.
 // (one 128-byte line per CTA: with the counters packed, the CTAs' polls queue up
 // on a few lines and a step's wait takes 4.5 us instead of 1.2).
-constexpr int HJ_SYNC_CTAS = 512;
+// One CTA per SM, of which there are 152.
+constexpr int HJ_SYNC_CTAS = 160;
 constexpr int HJ_SYNC_STRIDE = 32;
 struct HjResidentSync {
     unsigned int count;
@@ -174,7 +175,7 @@ struct hj_grid {
     } graphs[4];
     unsigned launch_version;  // bumped whenever a step kernel's parameters may change
     unsigned graph_tick;
-    HjResidentSync *rsync;    // resident kernel bookkeeping (allocated on first use)
+    HjResidentSync *rsync;    // resident and on-chip kernels' bookkeeping (behind *loop, in its allocation)
     size_t device_bytes;
 };
 
@@ -184,7 +185,7 @@ cudaError_t hj_launch_step_generic(hj_grid *g, long long n, int sel);
 cudaError_t hj_launch_step_tiled(hj_grid *g, long long n, int sel);
 // k steps from V after n steps in one cooperative launch of the resident
 // kernel, the last of them with dt[1] if cut (convergence mode: it stops early
-// when the test ends the loop); allocates g->rsync on first use.
+// when the test ends the loop).
 cudaError_t hj_launch_step_resident(hj_grid *g, long long n, long long k, bool cut);
 // The on-chip form of the resident kernel: choose the blocks for this grid
 // (oc_bx = 0: it does not take it), and its launch (as hj_launch_step_resident;

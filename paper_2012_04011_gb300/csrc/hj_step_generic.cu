@@ -914,14 +914,6 @@ bool hj_resident_supported(const hj_grid *g)
 
 cudaError_t hj_launch_step_resident(hj_grid *g, long long n, long long k, bool cut)
 {
-    if (!g->rsync) {
-        cudaError_t e = hj_malloc((void **)&g->rsync, sizeof(HjResidentSync));
-        if (e != cudaSuccess) {
-            g->rsync = nullptr;
-            return e;
-        }
-        g->device_bytes += sizeof(HjResidentSync);
-    }
     cudaError_t e = cudaMemsetAsync(g->rsync, 0, sizeof(HjResidentSync), g->stream);
     if (e != cudaSuccess) return e;
     if (!g->track && g->oc_bx > 0) return hj_launch_onchip(g, n, k, cut);

@@ -293,3 +293,17 @@ def test_resident_rejected_when_tables_do_not_fit(hj):
             g.set_kernel(hj.HJ_KERNEL_RESIDENT)
         assert e.value.status == hj.HJ_ERR_UNSUPPORTED
         assert g.info().kernel == hj.HJ_KERNEL_GENERIC
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "q527"])
+def test_solves_allocate_nothing(hj, prec):
+    """A grid's device memory is all there when it is created: the first solve
+    with the resident (or on-chip) kernel leaves it as it was."""
+    w = scenes.workload("car4d_31x31x11x16")
+    with hj.Grid.for_workload(w, prec_code(hj, prec)) as g:
+        g.set_kernel(hj.HJ_KERNEL_RESIDENT)
+        g.set_initial_value(scenes.initial_value(w.grid, w.scene))
+        before = g.info().device_bytes
+        g.solve_brt(w.T, w.cfl)
+        g.solve_converged(1e-3, 2 * w.T, w.cfl)
+        assert g.info().device_bytes == before
