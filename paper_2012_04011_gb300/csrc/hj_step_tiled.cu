@@ -104,36 +104,48 @@ int best_chunk(const hj_grid *g, int ncol, int slots)
 // an inner tile.  A plane of a tile at an end of v takes 1.7 + 0.5 / tv times as
 // long (extrapolated ghosts take the 64-bit form), at an end of y 1.1 times; the
 // CTAs take the items in next_item()'s order.  Beyond 16 rounds the CTAs' shares
-// are close to the mean, which is used instead.
-double heaviest_q527(const hj_grid *g, const TiledParams &P, int xc, int nchunk, int n)
+// are close to the mean, which is used instead.  Above `limit` the value is a
+// lower bound: the mean, or what a CTA has by then.
+double heaviest_q527(const hj_grid *g, const TiledParams &P, int xc, int nchunk, int n, double limit)
 {
     const long long items = (long long)P.ncol * nchunk;
-    double load[1024] = {0.0};
     const bool mean = items > 16LL * n || n > 1024;
     if (n > items) n = (int)items;
     const int ncol_y = P.ncol / P.ncol_v;
-    double sum = 0.0, most = 0.0;
+    const double end_v = 1.7 + 0.5 / P.tv;
+    auto planes_of = [&](int c) {
+        const int x0 = c * xc, x1 = x0 + xc < g->n[0] ? x0 + xc : g->n[0];
+        return (x1 < g->n[0] ? x1 + 1 : x1) - (x0 > 0 ? x0 - 1 : 0);
+    };
+    double planes = 0.0;
+    const bool alike = mean && nchunk > 4;  // (the inner chunks are)
+    for (int c = 0; c < (alike ? 3 : nchunk); ++c) planes += planes_of(c);
+    if (alike) planes *= (double)nchunk / 3;
+    // columns at an end of v, of those left at an end of y, inner ones
+    const int nv = P.ncol_v < 2 ? 1 : 2, ny = ncol_y < 2 ? 1 : 2, inner = P.ncol_v - nv;
+    const double share = planes * (ncol_y * nv * end_v + inner * (ny * 1.1 + (ncol_y - ny))) / n;
+    if (mean || share > limit) return share;
+    double load[1024] = {0.0}, most = 0.0;
     int shift = 0, place = 0;
     for (int c = 0; c < nchunk; ++c) {
-        const int x0 = c * xc, x1 = x0 + xc < g->n[0] ? x0 + xc : g->n[0];
-        const int planes = (x1 < g->n[0] ? x1 + 1 : x1) - (x0 > 0 ? x0 - 1 : 0);
-        for (int col = 0; col < P.ncol; ++col) {
-            const int iv = col % P.ncol_v, iy = col / P.ncol_v;
-            const bool end_v = iv == 0 || iv == P.ncol_v - 1, end_y = iy == 0 || iy == ncol_y - 1;
-            const double w = planes * (end_v ? 1.7 + 0.5 / P.tv : end_y ? 1.1 : 1.0);
-            sum += w;
-            if (!mean) most = fmax(most, load[(place + n - shift) % n] += w);
-            if (++place == n) {
-                place = 0;
-                shift = (shift + 1) % n;
+        const int np = planes_of(c);
+        for (int iy = 0; iy < ncol_y; ++iy) {
+            const double wy = np * (iy == 0 || iy == ncol_y - 1 ? 1.1 : 1.0), wv = np * end_v;
+            for (int iv = 0; iv < P.ncol_v; ++iv) {
+                const int cta = place >= shift ? place - shift : place + n - shift;
+                load[cta] += iv == 0 || iv == P.ncol_v - 1 ? wv : wy;
+                if (load[cta] > most) {
+                    most = load[cta];
+                    if (most > limit) return most;
+                }
+                if (++place == n) {
+                    place = 0;
+                    if (++shift == n) shift = 0;
+                }
             }
         }
-        if (mean && c == 2 && nchunk > 4) {  // the inner chunks are alike
-            sum *= (double)nchunk / 3;
-            break;
-        }
     }
-    return mean ? sum / n : most;
+    return most;
 }
 
 // Estimated time of a step (in us, up to what all shapes of a grid share) for
@@ -156,23 +168,67 @@ double heaviest_q527(const hj_grid *g, const TiledParams &P, int xc, int nchunk,
 // to 1.74 (1.22).  Per step, that rule and this one: 80x80x25x40 FP32 18.4 and
 // 15.4 us, 128x128x64x96 with the field 156 and 141, 128x128x30x16 with the
 // field 20.3 and 17.9.
-double step_cost(const hj_grid *g, const TiledParams &P, int slots, int xc_req)
+// A shape that a lower bound (no item order loads fewer planes than ncol n1 /
+// slots per CTA, none is cheaper than an inner one) shows to cost more than
+// `limit` returns that bound.
+double step_cost(const hj_grid *g, const TiledParams &P, int slots, int xc_req, double limit)
 {
     static const double F4D[4] = {0.0089, 0.0111, 0.0148, 0.0210}, FXY[4] = {0.0169, 0.0147, 0.0176, 0.0209},
                         Q[4] = {0.0326, 0.0300, 0.0296, 0.0357};
     const bool fixed = g->prec == HJ_Q527;
-    const int xc = xc_req > 0 && xc_req < g->n[0] ? xc_req : (xc_req > 0 ? g->n[0] : best_chunk(g, P.ncol, slots));
-    const int nchunk = (g->n[0] + xc - 1) / xc;
     int cls = 0;
     while (cls < 3 && P.nconsumer > hj_tiled_variant(fixed, cls)) ++cls;
     const double least = P.rpt > 1 ? 11 : 8, warps = P.nconsumer / 32 > least ? P.nconsumer / 32 : least;
+    double plane;  // time of a plane (fixed point: and `planes` times 0.25)
+    if (fixed) {
+        plane = warps * Q[cls];
+    } else if (!g->v0_bcast) {
+        plane = warps * F4D[cls] + 0.2875;
+    } else {
+        const double per_warp = P.rpt == 1 ? FXY[cls] : (P.rpt == 2 ? 2 * 0.0204 : 4 * 0.0152);
+        plane = warps * per_warp + 0.00497 * ((P.halo_box + g->p4 * P.ty * P.tv) / 256.0) + 0.1425;
+    }
+    const double bound = (1.0 - 1e-9) * P.ncol * g->n[0] / slots * (plane + (fixed ? 0.25 : 0.0));
+    if (bound > limit) return bound;
+    const int xc = xc_req > 0 && xc_req < g->n[0] ? xc_req : (xc_req > 0 ? g->n[0] : best_chunk(g, P.ncol, slots));
+    const int nchunk = (g->n[0] + xc - 1) / xc;
     const long long rounds = ((long long)P.ncol * nchunk + slots - 1) / slots;
     const double planes = (double)rounds * (xc + (nchunk > 1 ? 2 : 1));
-    if (fixed) return heaviest_q527(g, P, xc, nchunk, slots) * warps * Q[cls] + planes * 0.25;
-    if (!g->v0_bcast) return planes * (warps * F4D[cls] + 0.2875);
-    const double per_warp = P.rpt == 1 ? FXY[cls] : (P.rpt == 2 ? 2 * 0.0204 : 4 * 0.0152);
-    const double kb = (P.halo_box + g->p4 * P.ty * P.tv) / 256.0;
-    return planes * (warps * per_warp + 0.00497 * kb + 0.1425);
+    if (!fixed) return planes * plane;
+    const double rest = planes * 0.25;
+    return heaviest_q527(g, P, xc, nchunk, slots, (limit - rest) / plane) * plane + rest;
+}
+
+// The shape with the least step_cost() for a request that leaves one extent or
+// both (req[0], req[1] <= 0) open.  Large tiles first: they cost least on most
+// grids, and the others' bounds then show it (set-up of a Q5.27 grid of
+// 128x128x64x96 228 -> 143 us, 131 with the rule before step_cost(); of equal
+// shapes the smaller one counts).
+void default_shape(const hj_grid *g, int slots, int maxsmem, const int32_t *req, int *ty, int *tv)
+{
+    const bool fixed = g->prec == HJ_Q527;
+    const int cap = hj_tiled_variant(fixed, 2);
+    double best = 1e300;
+    int bty = 1, btv = 1;
+    for (int a = g->n[1] < 16 ? g->n[1] : 16; a >= 1; --a)
+        for (int b = g->n[2] < 16 ? g->n[2] : 16; b >= 1; --b) {
+            if ((req[0] > 0 && a != req[0]) || (req[1] > 0 && b != req[1])) continue;
+            const TiledParams C = make_params(g, a, b, 1, 0);
+            // (fixed point: tiles of one or two rows along an axis measured slower
+            // than the estimate, 70x90x40x72 69 us at 15 x 2, 61 at 6 x 5; an extent
+            // that is requested is taken as it is)
+            const bool thin = fixed && ((req[0] <= 0 && a < 3) || (req[1] <= 0 && b < 3));
+            const bool fits = !thin && C.nconsumer <= cap && 4 * (size_t)C.stage_bytes + 2048 <= (size_t)maxsmem;
+            if (!fits && !(a == 1 && b == 1)) continue;
+            const double c = fits ? step_cost(g, C, slots, req[2], best) : 1e299;
+            if (c <= best) {
+                best = c;
+                bty = a;
+                btv = b;
+            }
+        }
+    *ty = bty;
+    *tv = btv;
 }
 
 size_t tiled_smem_bytes(const TiledParams &P)
@@ -272,30 +328,7 @@ bool hj_tiled_setup(hj_grid *g, char *why, size_t why_len)
     if (max_consumers(fixed) / q4 < 1) return fail("theta rows too long for one CTA");
     const int32_t *req = g->tile_req[g->v0_bcast];
     int ty = req[0], tv = req[1];
-    if (ty <= 0 || tv <= 0) {
-        const int cap = hj_tiled_variant(fixed, 2);
-        double best = 1e300;
-        int bty = 1, btv = 1;
-        for (int a = 1; a <= 16 && a <= g->n[1]; ++a)
-            for (int b = 1; b <= 16 && b <= g->n[2]; ++b) {
-                if ((ty > 0 && a != ty) || (tv > 0 && b != tv)) continue;
-                const TiledParams C = make_params(g, a, b, 1, 0);
-                // (fixed point: tiles of one or two rows along an axis measured slower
-                // than the estimate, 70x90x40x72 69 us at 15 x 2, 61 at 6 x 5; an extent
-                // that is requested is taken as it is)
-                const bool thin = fixed && ((ty <= 0 && a < 3) || (tv <= 0 && b < 3));
-                const bool fits = !thin && C.nconsumer <= cap && 4 * (size_t)C.stage_bytes + 2048 <= (size_t)maxsmem;
-                if (!fits && !(a == 1 && b == 1)) continue;
-                const double c = fits ? step_cost(g, C, sms > 0 ? sms : 1, req[2]) : 1e299;
-                if (c < best) {
-                    best = c;
-                    bty = a;
-                    btv = b;
-                }
-            }
-        ty = bty;
-        tv = btv;
-    }
+    if (ty <= 0 || tv <= 0) default_shape(g, sms > 0 ? sms : 1, maxsmem, req, &ty, &tv);
     if (tv > g->n[2]) tv = g->n[2];
     if (ty > g->n[1]) ty = g->n[1];
     while (consumers_of(g, ty, tv) > max_consumers(fixed) && ty > 1) --ty;
