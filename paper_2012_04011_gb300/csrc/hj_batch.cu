@@ -632,6 +632,7 @@ struct SlotHost {
     bool has_value = false;
     double T = 0, cfl = 0.8;
     int ty = 0, tv = 0, xc = 0;
+    int tile[3][2] = {};  // the tile for B_VARIANTS[0..2] consumers (rows along y and v; 0: not chosen yet)
     HjGeom geom;
 };
 
@@ -841,6 +842,74 @@ hj_status upload_slot_tables(hj_batch *b, SlotHost &s)
     return HJ_OK;
 }
 
+// Resident CTAs of a block of nc consumers (before the occupancy query).
+long long resident_ctas(const hj_batch *b, int nc) { return (long long)b->sms * (nc <= B_DUAL ? 2 : 1); }
+
+// x chunks per column of a layout of `columns` columns on `ctas` CTAs, and the
+// planes of one.
+int chunk_count(const hj_batch *b, long long columns, int min_n1, long long ctas)
+{
+    if (b->xc_mode > 0) return b->xc_mode;
+    if (columns < 1 || columns >= ctas) return 1;
+    const int most = min_n1 / 4 > 1 ? min_n1 / 4 : 1;  // chunks of at least 4 planes
+    const long long want = (ctas + columns - 1) / columns;
+    return want < most ? (int)want : most;
+}
+int chunk_planes(int n1, int nchunk)
+{
+    const int xc = (n1 + nchunk - 1) / nchunk;
+    return xc >= 4 ? xc : (n1 < 4 ? n1 : 4);
+}
+
+// Consumers of the automatic shape: of 352, 480 and 608 the one with the least
+//     (planes per CTA + planes of the longest slot step + 12) (1 + 0.09 warps),
+// the time of a batch step in units of a plane's fixed part: a round of the
+// queue takes each CTA its share, and a slot's next step waits for the last of
+// its items.  Larger blocks have fewer items, but of a longer plane.  The two
+// constants are fitted to 840 random batches (1 to 64 slots of 20x20x9x8 to
+// 100x100x32x128).  On 400 others, against the first rule (352 up to 44 headings,
+// 480 up to 60, 608, 736 beyond): mean time 0.945, 17 slower by more than 2 %, 2
+// by more than 5 %; 480 always: 0.959, 72 and 45.  (64 slots of up to
+// 60x60x24x36 take 480: 22.4 ms per solve through the API, 26.5 with 352.)
+int auto_consumers(hj_batch *b)
+{
+    const int order[3] = {1, 0, 2};
+    int best_nc = B_VARIANTS[1];
+    double best = 1e300;
+    for (int v : order) {
+        const int nc = B_VARIANTS[v];
+        long long columns = 0;
+        int min_n1 = 1 << 30, warps = 1;
+        for (SlotHost &s : b->slots) {
+            if (!s.used) continue;
+            int *t = s.tile[v];
+            if (t[0] == 0) choose_tile(s, nc, &t[0], &t[1]);
+            columns += (long long)((s.n[1] + t[0] - 1) / t[0]) * ((s.n[2] + t[1] - 1) / t[1]);
+            if (s.n[0] < min_n1) min_n1 = s.n[0];
+            const int w = ((s.p4 / 4) * t[0] * t[1] + 31) / 32;
+            if (w > warps) warps = w;
+        }
+        const long long ctas = resident_ctas(b, nc);
+        const int nchunk = chunk_count(b, columns, min_n1, ctas);
+        double share = 0.0, longest = 0.0;
+        for (SlotHost &s : b->slots) {
+            if (!s.used) continue;
+            const int xc = chunk_planes(s.n[0], nchunk), nch = (s.n[0] + xc - 1) / xc;
+            const long long items = (long long)nch * ((s.n[1] + s.tile[v][0] - 1) / s.tile[v][0]) *
+                                    ((s.n[2] + s.tile[v][1] - 1) / s.tile[v][1]);
+            const double planes = (double)(s.n[0] + 2 * (nch - 1)) / nch;
+            share += items * planes / ctas;
+            longest = fmax(longest, planes * ((items + ctas - 1) / ctas));
+        }
+        const double c = (share + longest + 12.0) * (1.0 + 0.09 * warps);
+        if (c < best) {
+            best = c;
+            best_nc = nc;
+        }
+    }
+    return best_nc;
+}
+
 // Item layout of the slots marked in `active` for `ctas` resident CTAs (the
 // tiles chosen by rebuild): x chunks per slot, h_insts' xc and nitems
 // (0 for the others), and the queue in order.  Whole columns while the
@@ -867,12 +936,7 @@ void plan_layout(hj_batch *b, const std::vector<char> &active, const std::vector
         if (s.n[0] < min_n1) min_n1 = s.n[0];
         order.push_back(i);
     }
-    int nchunk = b->xc_mode > 0 ? b->xc_mode : 1;
-    if (b->xc_mode == 0 && columns > 0 && columns < ctas) {
-        nchunk = (int)((ctas + columns - 1) / columns);
-        const int most = min_n1 / 4 > 1 ? min_n1 / 4 : 1;  // chunks of at least 4 planes
-        if (nchunk > most) nchunk = most;
-    }
+    const int nchunk = chunk_count(b, columns, min_n1, ctas);
     // slots with more steps to go first (a launch's later rounds are then a
     // prefix of the list), then the longest columns first
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
@@ -882,8 +946,7 @@ void plan_layout(hj_batch *b, const std::vector<char> &active, const std::vector
     std::vector<int> slot_chunks(b->max_slots, nchunk);
     for (int i : order) {
         SlotHost &s = b->slots[i];
-        s.xc = (s.n[0] + slot_chunks[i] - 1) / slot_chunks[i];
-        if (s.xc < 4) s.xc = s.n[0] < 4 ? s.n[0] : 4;
+        s.xc = chunk_planes(s.n[0], slot_chunks[i]);
         const int ncv = (s.n[2] + s.tv - 1) / s.tv, ncy = (s.n[1] + s.ty - 1) / s.ty;
         const int nch = (s.n[0] + s.xc - 1) / s.xc;
         b->h_insts[i].xc = s.xc;
@@ -896,21 +959,13 @@ void plan_layout(hj_batch *b, const std::vector<char> &active, const std::vector
     b->lay_order = order;
 }
 
-// Resident CTAs of a block of nc consumers (before the occupancy query).
-long long resident_ctas(const hj_batch *b, int nc) { return (long long)b->sms * (nc <= B_DUAL ? 2 : 1); }
-
 // Rebuild the per-slot descriptors, tensor maps and item list after slots or
 // the kernel shape changed.
 hj_status rebuild(hj_batch *b)
 {
     BEncodeFn enc = batch_encode_fn();
     if (!enc) return bfail(HJ_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
-    // block size: the request, else 480 consumers.  Device ms of whole solves with
-    // 288 (two CTAs per SM), 352 and 480 consumers: 64 slots of up to 60x60x24x36
-    // 19.4, 22.8, 19.7; 16 of them 6.1, 6.3, 5.5; 4 of them 2.27, 2.23, 2.38; eight
-    // of 31x31x11x16 to 100x100x30x48 5.3, 5.7, 4.9; one of 128x128x64x96 (18 steps)
-    // 4.3, 4.0, 3.6.
-    const int nc = b->nconsumer_req > 0 ? b->nconsumer_req : B_VARIANTS[1];
+    const int nc = b->nconsumer_req > 0 ? b->nconsumer_req : auto_consumers(b);
     b->h_insts.assign(b->max_slots, BatchInst());
     std::vector<BatchInst> &insts = b->h_insts;
     std::vector<CUtensorMap> maps((size_t)4 * b->max_slots);

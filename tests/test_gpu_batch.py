@@ -286,6 +286,7 @@ def test_a_later_batch_does_not_lower_the_shared_memory_limit(hj):
     v0s = [scenes.initial_value(w.grid, w.scene) for w in ws]
     with hj.Batch(1) as a, hj.Batch(1) as b:
         for bt, w in ((a, ws[0]), (b, ws[1])):
+            bt.set_shape(480, 0)
             bt.add_workload(w)
         for k in (0, 1, 0):
             bt = (a, b)[k]
@@ -293,3 +294,22 @@ def test_a_later_batch_does_not_lower_the_shared_memory_limit(hj):
             bt.set_horizon(0, ws[k].T, ws[k].cfl)
             assert bt.advance().finished == 1
             assert np.array_equal(bt.read_value(0), single_grid(hj, ws[k], v0s[k])[0])
+
+
+@pytest.mark.parametrize("n, slots, tile", [((30, 14, 6, 30), 2, (7, 6)), ((12, 60, 20, 36), 16, (5, 10)),
+                                            ((12, 40, 20, 72), 16, (8, 4))])
+def test_batch_default_shape_follows_the_slots(hj, n, slots, tile):
+    """The automatic shape: 352 consumers where few items leave a step as long
+    as its longest one, 480 and 608 where more rows per item save some; the
+    slots give the single-grid results with each."""
+    ws = [scenes.custom_workload(n, n_circles=2, n_rects=1, T=0.2, seed=60 + i) for i in range(slots)]
+    v0s = [scenes.initial_value(w.grid, w.scene) for w in ws]
+    with hj.Batch(slots) as b:
+        for k, (w, v0) in enumerate(zip(ws, v0s)):
+            assert b.add_workload(w) == k
+            b.set_initial_value(k, v0)
+            b.set_horizon(k, w.T, w.cfl)
+        assert b.advance().finished == slots
+        for k in (0, slots // 2, slots - 1):
+            assert tuple(b.slot_info(k).tile)[:2] == tile
+            assert np.array_equal(b.read_value(k), single_grid(hj, ws[k], v0s[k])[0])
