@@ -534,6 +534,11 @@ HJ_API hj_status hj_wait_selftest(int64_t limit_ns, int32_t *status, int64_t *wa
  * side effects as hj_wait_selftest. */
 HJ_API hj_status hj_barrier_selftest(int64_t limit_ns, int32_t *status, int64_t *waited_ns);
 
+/* The same self-test for the waits between neighbouring blocks of the on-chip
+ * form of HJ_KERNEL_RESIDENT: one CTA waits, with that kernel's bounded wait,
+ * for a step that no neighbour publishes. */
+HJ_API hj_status hj_neighbour_selftest(int64_t limit_ns, int32_t *status, int64_t *waited_ns);
+
 /* Test of a step launch that fails: of the step launches that follow on g
  * (one per step; one per call of HJ_KERNEL_RESIDENT), number `launch` (1, 2,
  * ...; 0: none) fails on the host without being made.  The call that meets it

@@ -9,13 +9,15 @@
 // record the status.  Nothing faults, traps or hangs; the context stays
 // usable.  The grid-barrier self-test does the same for the resident step
 // kernel's barrier (hj_grid_sync): two co-resident CTAs wait for a third
-// arrival that never comes.
+// arrival that never comes.  The neighbour self-test does it for the on-chip
+// kernel's wait (wait_published): a CTA that finds its neighbour's first step
+// published waits for the second, which never is.
 //
 // Also here: the FP64 fused multiply-add throughput probe that the FP64
 // roofline of the FP64 step kernel and of the query kernel is measured
 // against (GB300's FP64 rate is a small fraction of its FP32 rate, so the
 // measured figure, not a nominal one, is the denominator).
-#include "hj_resident.cuh"
+#include "hj_onchip.cuh"
 
 namespace {
 
@@ -76,6 +78,30 @@ __global__ void barrier_selftest_kernel(HjResidentSync *sync, unsigned long long
     }
 }
 
+// The two polling threads of one CTA: neighbour 0 has published step 1, and
+// nobody publishes step 2.
+__global__ void neighbour_selftest_kernel(HjResidentSync *sync, unsigned long long limit_ns, int *status,
+                                          unsigned long long *waited_ns)
+{
+    __shared__ int s_ok;
+    if (threadIdx.x == 0) {
+        s_ok = 1;
+        sync->prog[0] = 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    const unsigned long long t0 = global_ns();
+    if (threadIdx.x < 2) {
+        if (!hj_onchip::wait_published(sync->prog, 1u, limit_ns)) s_ok = -1;  // this one is there
+        else if (!hj_onchip::wait_published(sync->prog, 2u, limit_ns)) s_ok = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s_ok == 0) atomicExch(status, (int)HJ_ERR_TIMEOUT);
+        *waited_ns = global_ns() - t0;
+    }
+}
+
 typedef void (*SelftestLaunch)(unsigned long long limit_ns, int *status, unsigned long long *waited_ns, void *scratch,
                                cudaError_t *err);
 
@@ -93,7 +119,7 @@ hj_status run_selftest(int64_t limit_ns, int32_t *status, int64_t *waited_ns, Se
         return HJ_ERR_INVALID_ARG;
     }
     char *d = nullptr;
-    const size_t bytes = 16 + sizeof(HjResidentSync);
+    const size_t bytes = 128 + sizeof(HjResidentSync);
     cudaError_t e = hj_malloc((void **)&d, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();  // the failed allocation must not fail later launch checks
@@ -103,7 +129,7 @@ hj_status run_selftest(int64_t limit_ns, int32_t *status, int64_t *waited_ns, Se
     int *d_status = (int *)d;
     unsigned long long *d_waited = (unsigned long long *)(d + 8);
     e = cudaMemset(d, 0, bytes);
-    if (e == cudaSuccess) launch((unsigned long long)limit_ns, d_status, d_waited, d + 16, &e);
+    if (e == cudaSuccess) launch((unsigned long long)limit_ns, d_status, d_waited, d + 128, &e);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     int h_status = -1;
     unsigned long long h_waited = 0;
@@ -133,7 +159,19 @@ void launch_barrier(unsigned long long limit_ns, int *status, unsigned long long
     *err = cudaLaunchCooperativeKernel((const void *)barrier_selftest_kernel, 2, 64, args, 0, 0);
 }
 
+void launch_neighbour(unsigned long long limit_ns, int *status, unsigned long long *waited_ns, void *scratch,
+                      cudaError_t *err)
+{
+    neighbour_selftest_kernel<<<1, 64>>>((HjResidentSync *)scratch, limit_ns, status, waited_ns);
+    *err = cudaGetLastError();
+}
+
 }  // namespace
+
+extern "C" hj_status hj_neighbour_selftest(int64_t limit_ns, int32_t *status, int64_t *waited_ns)
+{
+    return run_selftest(limit_ns, status, waited_ns, launch_neighbour);
+}
 
 extern "C" hj_status hj_barrier_selftest(int64_t limit_ns, int32_t *status, int64_t *waited_ns)
 {

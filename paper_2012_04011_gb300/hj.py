@@ -162,6 +162,8 @@ _SIGS = {
                                         ctypes.POINTER(ctypes.c_int64)]),
     "hj_barrier_selftest": (ctypes.c_int, [ctypes.c_int64, ctypes.POINTER(ctypes.c_int32),
                                            ctypes.POINTER(ctypes.c_int64)]),
+    "hj_neighbour_selftest": (ctypes.c_int, [ctypes.c_int64, ctypes.POINTER(ctypes.c_int32),
+                                             ctypes.POINTER(ctypes.c_int64)]),
     "hj_launch_selftest": (ctypes.c_int, [_VP, ctypes.c_int64]),
     "hj_stop_selftest": (ctypes.c_int, [_VP, ctypes.c_double, ctypes.c_double, ctypes.c_double,
                                         ctypes.POINTER(ctypes.c_int32)]),
@@ -374,6 +376,14 @@ def hj_barrier_selftest(limit_ns: int):
     st = ctypes.c_int32(0)
     waited = ctypes.c_int64(0)
     _check(lib.hj_barrier_selftest(int(limit_ns), ctypes.byref(st), ctypes.byref(waited)))
+    return int(st.value), int(waited.value)
+
+
+def hj_neighbour_selftest(limit_ns: int):
+    """(status, waited_ns) of the bounded wait between blocks of the on-chip kernel."""
+    st = ctypes.c_int32(0)
+    waited = ctypes.c_int64(0)
+    _check(lib.hj_neighbour_selftest(int(limit_ns), ctypes.byref(st), ctypes.byref(waited)))
     return int(st.value), int(waited.value)
 
 

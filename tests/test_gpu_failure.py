@@ -82,3 +82,25 @@ def test_fp64_probe_counts_and_runs(hj):
     assert n == sms * 8 * 256 * 8 * iters
     tflops = 2.0 * n / (e0.elapsed_time(e1) * 1e-3) / 1e12
     assert 0.05 < tflops < 10.0, tflops
+
+
+def test_neighbour_wait_times_out_and_context_survives(hj):
+    """The on-chip kernel's wait for its neighbours: a published step is seen at
+    once, one that nobody publishes ends at the limit."""
+    status, waited = hj.hj_neighbour_selftest(50_000_000)  # 50 ms
+    assert status == hj.HJ_ERR_TIMEOUT
+    assert 50_000_000 <= waited < 1_000_000_000
+    with pytest.raises(hj.HjError) as e:
+        hj.hj_neighbour_selftest(10)
+    assert e.value.status == hj.HJ_ERR_INVALID_ARG
+    # an on-chip solve on the same context completes and matches the oracle's codes
+    w = scenes.workload("car4d_31x31x11x16")
+    V0 = scenes.initial_value(w.grid, w.scene)
+    with hj.Grid.for_workload(w, hj.HJ_Q527) as g:
+        g.set_kernel(hj.HJ_KERNEL_RESIDENT)
+        g.set_initial_value(V0)
+        g.solve_brt(w.T, w.cfl)
+        V = g.read_value()
+    P = oracle.Problem(w.grid.n, w.grid.lo, w.grid.hi, w.grid.periodic, oracle.DYN_CAR4D, (w.a_max, w.w_max))
+    Q, _ = oracle.solve_q527(P, V0, w.T, w.cfl, nthreads=oracle.max_threads())
+    assert np.array_equal(V, Q / 2.0 ** 27)
