@@ -307,3 +307,35 @@ def test_solves_allocate_nothing(hj, prec):
         g.solve_brt(w.T, w.cfl)
         g.solve_converged(1e-3, 2 * w.T, w.cfl)
         assert g.info().device_bytes == before
+
+
+@pytest.mark.parametrize("prec", ["fp32", "q527"])
+@pytest.mark.parametrize("n", [(100, 100, 25, 30), (97, 90, 23, 27), (96, 90, 22, 29), (95, 88, 26, 28)])
+@pytest.mark.parametrize("lo_v", [0.0, -2.5])
+def test_resident_off_chip_padded_rows(hj, n, prec, lo_v):
+    """Grids of more values than the SMs' shared memory holds twice (4.4 M), so
+    that the L2-resident form runs, with rows padded by one, two, three and no
+    lanes: bit for bit against the generic kernel, in one call and in pieces
+    that start in either buffer."""
+    assert n[0] * n[1] * n[2] * ((n[3] + 3) // 4 * 4) * 8 > 152 * 227 * 1024
+    lo = (-5.0, -5.0, lo_v, -np.pi)
+    grid = scenes.GridSpec(n, lo)
+    rng = np.random.default_rng(sum(n))
+    V0 = scenes.initial_value(grid, scenes.random_scene(rng, 3)) + 0.05 * rng.standard_normal(n)
+    out = []
+    for kernel, chunk in ((hj.HJ_KERNEL_GENERIC, 1 << 40), (hj.HJ_KERNEL_RESIDENT, 1 << 40),
+                          (hj.HJ_KERNEL_RESIDENT, 3)):
+        with hj.Grid(n, lo, grid.hi, grid.periodic, prec_code(hj, prec)) as g:
+            g.set_dynamics(hj.HJ_DYN_CAR4D, (scenes.A_MAX, scenes.W_MAX))
+            g.set_kernel(kernel)
+            g.set_initial_value(V0)
+            steps = 0
+            while True:
+                st = g.advance_brt(0.12, scenes.CFL, chunk)
+                steps += st.steps
+                if st.t_final == 0.12:
+                    break
+            assert st.kernel == kernel and steps > 4
+            out.append((read_raw(hj, g, prec), steps))
+    for V, steps in out[1:]:
+        assert steps == out[0][1] and np.array_equal(V, out[0][0])
