@@ -10,7 +10,8 @@ FP32 cell-update: read V_n, read V0, write V_{n+1}).
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
 Under torchrun (N > 1) every rank solves its own replica (no data-path
-collective); the JSON line reports the whole-job rate.  --impl reference
+collective); the JSON line (the last one; the one before it, "detail ...", holds
+every other path's figures) reports the whole-job rate.  --impl reference
 times the FP64 CPU oracle on a bounded sample of the same workload.
 """
 from __future__ import annotations
@@ -830,10 +831,26 @@ def run_ours(args):
             "value": rate1, "unit": UNIT, "cores": 1, "kind": "oracle",
             "sample": f"{nst1} oracle time step of the {WORKLOAD} solve ({nst1 * ncell:.3e} cell-updates, "
                       f"{el1:.1f} s), FP64, one thread"}
-    print(json.dumps(line, default=json_default), flush=True)
+    print("detail " + json.dumps(line, default=json_default), flush=True)
+    print(json.dumps(headline(line), default=json_default), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
     return 0
+
+
+# What the last line of the output holds: the run's result, short enough to be
+# read whole where only the end of an output is kept.  The line before it holds
+# the rest: every path's figures, the shapes tried, the serving sweep.
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "roofline", "latency_ms", "clocks", "gpu_launches", "e2e")
+
+
+def headline(line):
+    out = {k: line[k] for k in HEADLINE if k in line}
+    out["config"] = dict(out["config"])
+    if out["config"].get("tile"):
+        out["config"]["tile"] = {k: v for k, v in out["config"]["tile"].items() if k != "tried"}
+    return out
 
 
 def json_default(o):
