@@ -121,7 +121,8 @@ typedef enum {
                             * cooperative launch with a grid barrier between steps, or, for FP32
                             * and Q5.27 car grids that fit, with the values held in the SMs'
                             * shared memory and waits between neighbouring blocks only; a wait
-                            * that runs out (2 s) ends the call with HJ_ERR_TIMEOUT */
+                            * that runs out (2 s) ends the call with HJ_ERR_TIMEOUT (and the value is
+                            * lost: HJ_ERR_STATE from reads and queries until the next V0) */
 } hj_kernel;
 
 typedef struct {
@@ -388,8 +389,9 @@ HJ_API hj_status hj_batch_add(hj_batch *b, const int32_t n[4], const double lo[4
                               const double params[2], int32_t *slot);
 
 /* Free a slot.  Its device memory returns to the budget; the batch keeps up
- * to 1 GiB of such memory, the latest freed, for new slots of the same sizes,
- * until it is destroyed or another allocation of this library needs it. */
+ * to 1 GiB of such memory for new slots of the same sizes, until it is
+ * destroyed, another allocation of this library needs it, or other sizes have
+ * taken its place. */
 HJ_API hj_status hj_batch_remove(hj_batch *b, int32_t slot);
 
 /* V0 of a slot from a host FP64 array or a device FP32/FP64 array (layout as

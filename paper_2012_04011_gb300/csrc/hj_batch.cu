@@ -55,6 +55,8 @@ constexpr int B_DUAL = 288;
 constexpr int B_MAX_ROUNDS = 1024;
 // Memory of removed slots a batch keeps at most.
 constexpr size_t B_POOL_BYTES = 1ull << 30;
+// Slots added since such a block was kept after which it makes room for others.
+constexpr long long B_POOL_STALE = 64;
 
 struct BatchInst {
     int n1, n2, n3, n4, p4, q4;
@@ -645,7 +647,13 @@ struct hj_batch {
     // served request costs an allocation and a free otherwise): at most
     // B_POOL_BYTES, within the budget together with the slots in use, and given
     // up when an allocation of the library finds the device out of memory
-    std::vector<std::pair<void *, size_t>> pool;
+    struct Kept {
+        void *mem;
+        size_t bytes;
+        long long added;  // slots added to the batch by then
+    };
+    std::vector<Kept> pool;  // oldest first
+    long long added = 0;
     size_t pool_bytes = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -724,20 +732,21 @@ void shrink_pool(hj_batch *b, size_t keep)
 {
     size_t k = 0;
     for (; k < b->pool.size() && b->pool_bytes > keep; ++k) {
-        cudaFree(b->pool[k].first);
-        b->pool_bytes -= b->pool[k].second;
+        cudaFree(b->pool[k].mem);
+        b->pool_bytes -= b->pool[k].bytes;
     }
     b->pool.erase(b->pool.begin(), b->pool.begin() + k);
 }
 
-// Device memory of a new slot: a kept block of that size, else a fresh one.
+// Device memory of a new slot: the latest kept block of that size, else a fresh one.
 cudaError_t slot_alloc(hj_batch *b, size_t bytes, void **mem)
 {
     {
         std::lock_guard<std::mutex> lock(pool_mutex());
-        for (size_t i = 0; i < b->pool.size(); ++i)
-            if (b->pool[i].second == bytes) {
-                *mem = b->pool[i].first;
+        ++b->added;
+        for (size_t i = b->pool.size(); i-- > 0;)
+            if (b->pool[i].bytes == bytes) {
+                *mem = b->pool[i].mem;
                 b->pool_bytes -= bytes;
                 b->pool.erase(b->pool.begin() + i);
                 return cudaSuccess;
@@ -749,19 +758,22 @@ cudaError_t slot_alloc(hj_batch *b, size_t bytes, void **mem)
 }
 
 // Memory of a removed slot (no longer in used_bytes; the stream is idle): kept
-// in place of the oldest blocks, so that the sizes served now are the ones
-// that find a block.
+// if there is room, or room can be made by freeing blocks that no slot has
+// needed for a while.  (Room is not made at the expense of sizes that are being
+// served: a large block would push out many small ones, and each cudaFree waits
+// for the device.)
 void slot_free(hj_batch *b, void *mem, size_t bytes)
 {
     std::lock_guard<std::mutex> lock(pool_mutex());
     const size_t left = b->budget > b->used_bytes ? b->budget - b->used_bytes : 0;
     const size_t cap = left < B_POOL_BYTES ? left : B_POOL_BYTES;
-    if (bytes > cap) {
+    while (b->pool_bytes + bytes > cap && !b->pool.empty() && b->added - b->pool[0].added > B_POOL_STALE)
+        shrink_pool(b, b->pool_bytes - 1);  // (the oldest one)
+    if (b->pool_bytes + bytes > cap) {
         cudaFree(mem);
         return;
     }
-    shrink_pool(b, cap - bytes);
-    b->pool.push_back({mem, bytes});
+    b->pool.push_back({mem, bytes, b->added});
     b->pool_bytes += bytes;
 }
 

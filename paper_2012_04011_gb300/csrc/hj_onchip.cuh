@@ -14,10 +14,10 @@
 // theta neighbours outside the quad a warp shuffle (shared memory where the
 // row or the warp ends).  V is held twice (before and after the step).  The
 // sweep is bound by shared-memory bandwidth and issue (about 31 shared-memory
-// wavefronts and 130 instructions per warp and column).  Measured, us per step
-// with the L2-resident form and with this one: 31x31x11x16 FP32 4.2 -> 2.4,
-// 60x60x20x36 FP32 12.1 -> 5.3, Q5.27 with steering 18.1 -> 8.5, 47x53x17x27
-// with steering 9.0 -> 4.0.  What was tried and is slower: V and V0 in registers
+// wavefronts and 190 instructions per warp and column).  Measured, us per step
+// with the L2-resident form and with this one: 31x31x11x16 FP32 3.2 -> 2.4,
+// 60x60x20x36 FP32 10.9 -> 5.3, Q5.27 with steering 16.5 -> 8.5, 47x53x17x27
+// with steering 6.5 -> 4.0.  What was tried and is slower: V and V0 in registers
 // with the columns unrolled (spills, and 240 instructions per column: 9.5 us on
 // 60x60x20x36), the paired FP32 instructions (fewer instructions, but each
 // takes two turns of the FMA pipe: 39 against 33 clocks per warp and column).
@@ -32,8 +32,8 @@
 // s + 1 only after its neighbours have published step s, that is, after they
 // have read what it overwrites.  Only neighbours wait for one another: there
 // is no grid-wide barrier.  Every wait is bounded (limit_ns); on timeout the
-// CTA records HJ_ERR_TIMEOUT and leaves, and its neighbours' waits run out in
-// turn.
+// CTA records HJ_ERR_TIMEOUT and leaves, and its neighbours, which wait for its
+// step since at most a step's time, run out with it.
 //
 // The per-cell arithmetic is the resident and generic kernels' (cell_value,
 // hj_q527_update), in the same order: the results are the same bit for bit.

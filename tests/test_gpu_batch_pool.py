@@ -61,10 +61,11 @@ def test_kept_memory_follows_the_sizes_that_are_served(hj):
     with hj.Batch(2, memory_budget=1 << 32) as b:
         free = lambda: torch.cuda.mem_get_info()[0]  # noqa: E731
         add_and_remove(b, old)
-        add_and_remove(b, new)
+        for _ in range(70):  # the first size is not asked for again
+            add_and_remove(b, new)
         before = free()
         slot = b.add_workload(scenes.custom_workload(new, n_circles=1, T=0.1, seed=1))
-        assert before - free() < 64 * MB  # the block of that size was there
+        assert before - free() < 64 * MB  # a block of that size was there
         b.remove(slot)
         # never more than 1 GiB is kept
         for k in range(4):
