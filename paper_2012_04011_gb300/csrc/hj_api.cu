@@ -1416,6 +1416,9 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
             if ((r = launch_step(g, HJ_KERNEL_TILED, i, 0)) != HJ_OK) return r;
         HJ_CUDA(cudaEventRecord(g->ev[2], g->stream));
         HJ_CUDA(cudaEventSynchronize(g->ev[2]));
+        if (read_status(g) != HJ_OK)
+            return set_err((hj_status)read_status(g), "device reported %s during autotune",
+                           hj_status_string((hj_status)read_status(g)));
         return HJ_OK;
     };
     double best = 1e300;
@@ -1434,11 +1437,6 @@ hj_status hj_autotune(hj_grid *g, int32_t steps_per_trial, hj_tile_result *resul
             else if (g->tile_xc == auto_xc) continue;  // the automatic choice already was one chunk
             if ((s = run_steps(2)) != HJ_OK) break;  // warm-up
             if ((s = run_steps(steps_per_trial)) != HJ_OK) break;
-            if (read_status(g) != HJ_OK) {
-                s = set_err((hj_status)read_status(g), "device reported %s during autotune",
-                            hj_status_string((hj_status)read_status(g)));
-                break;
-            }
             float ms = 0.f;
             cudaEventElapsedTime(&ms, g->ev[1], g->ev[2]);
             const double per = ms / steps_per_trial;

@@ -164,3 +164,26 @@ def test_steps_behind_a_timed_out_one_leave_at_once(hj, prec, xy, threshold, n):
         g.set_initial_value(V0)
         g.solve_brt(w.T, w.cfl)
         assert np.array_equal(g.read_value(), out[0])
+
+
+@pytest.mark.parametrize("launch", [1, 7, 60])
+def test_failed_autotune_at_any_trial_leaves_status_and_steps(hj, launch):
+    """A launch that fails in the first trial, in a later one, and (if there are
+    so many) among the re-timed shapes: the grid then solves as a new one."""
+    w = scenes.custom_workload((40, 41, 16, 24), n_circles=3, T=0.3, seed=11)
+    V0 = scenes.initial_value(w.grid, w.scene)
+    out = []
+    for tuned in (False, True):
+        with hj.Grid.for_workload(w, hj.HJ_FP32) as g:
+            g.set_kernel(hj.HJ_KERNEL_TILED)
+            g.set_initial_value(V0)
+            if tuned:
+                hj.hj_launch_selftest(g.handle, launch)
+                try:
+                    g.autotune(2)
+                except hj.HjError as e:
+                    assert e.status == hj.HJ_ERR_CUDA
+                hj.hj_launch_selftest(g.handle, 0)
+            st = g.solve_brt(w.T, w.cfl)
+            out.append((g.read_value(), st.steps, st.t_final))
+    assert out[0][1:] == out[1][1:] and np.array_equal(out[0][0], out[1][0])
