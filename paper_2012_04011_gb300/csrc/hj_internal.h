@@ -141,7 +141,7 @@ struct hj_grid {
     double t;              // simulated time
     long long nstep;       // steps since V0 was set
     double alpha[4];       // alpha_d^max of the current dynamics (over the grid's (v, theta) states)
-    double up_dt[2];       // step sizes the device constants and dt-scaled tables hold (0: none)
+    double up_dt[2];       // step sizes the device constants and dt-scaled tables hold (negative: none)
 
     bool has_dyn, has_value;
     bool value_lost;       // no value because a call failed after steps had run that it could not count

@@ -157,13 +157,14 @@ double heaviest_q527(const hj_grid *g, const TiledParams &P, int xc, int nchunk,
 // is latency-bound and a plane takes as long as with that many.  In fixed
 // point the tiles' costs differ and the CTA with the heaviest items sets the
 // time.  Coefficients: least squares over the 20 to 40 shapes that
-// hj_autotune timed on each of 10 grids (2 to 101 M cells; 18 in fixed point).
+// hj_autotune timed on each of 10 grids (2 to 101 M cells; 18 in fixed point):
+// the FP32 ones of the present kernels, the fixed-point ones of the kernel
+// before a warp took one form of the update.
 // Against the best timed shape of each grid the picks take 1.00 to 1.03 times
 // as long with a 4D V0 (mean 1.01), 1.00 to 1.11 (1.02; 6 of the 16 grids not
-// in the fit) with the field and 1.00 to 1.18 (1.04) in fixed point (fitted
-// when a warp with and without ghosts ran both forms, 1.00 to 1.11 then; a fit
-// to the present kernel with the 736 class gained up to 15 % on 7 of the 18
-// grids and lost up to 14 % on 4); the shape with the fewest halo reads per
+// in the fit) with the field and 1.00 to 1.18 (1.04) in fixed point (1.00 to
+// 1.11 with the kernel of the fit; a fit to the present kernel with the 736
+// class gained up to 15 % on 7 of the 18 grids and lost up to 14 % on 4); the shape with the fewest halo reads per
 // row, the rule before, took 1.00 to 1.33 (1.13), 1.03 to 1.26 (1.16) and 1.00
 // to 1.74 (1.22).  Per step, that rule and this one: 80x80x25x40 FP32 18.4 and
 // 15.4 us, 128x128x64x96 with the field 156 and 141, 128x128x30x16 with the
